@@ -207,7 +207,8 @@ int sv_set_wait_limit(sv_solver* s, int polls);
  *     budget of 3 blocks/SM (default), 2 or 4 blocks/SM, 1024-cell tiles with
  *     two cell pairs per thread, or warps sliding over 64-cell chunks (the
  *     kernel of every other 1D solver, its only config);
- *   2D / 3D: planes per block along the marching axis, 64 / 128 / 256 / 512.
+ *   2D / 3D: at most 64 / 128 / 256 / 512 planes per block along the marching
+ *     axis (fewer where a small grid would otherwise not fill the device).
  * sv_autotune times each configuration on the solver's current state and
  * keeps the fastest; the state, time and status are restored afterwards.
  * ------------------------------------------------------------------------ */

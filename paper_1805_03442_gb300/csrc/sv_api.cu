@@ -22,7 +22,7 @@ using namespace sv;
 // One launch configuration of a solver's per-step kernel (sv_set_config).
 struct SolverConfig {
   int kind;        // CFG_TILE, CFG_SLIDE or CFG_ND
-  int param;       // TILE: 10 x cell pairs per thread + blocks per SM; ND: planes per segment
+  int param;       // TILE: 10 x cell pairs per thread + blocks per SM; ND: planes per segment at most
   const char* desc;
 };
 enum { CFG_TILE = 0, CFG_SLIDE = 1, CFG_ND = 2 };
@@ -48,6 +48,7 @@ struct sv_solver {
   double* host_sums = nullptr;
   int grid = 0;
   int tile_grid = 0;                   // grid of the block-tile kernel of the current config
+  int nseg = 1;                        // 2D / 3D: segments of the marching axis (current config)
   std::vector<SolverConfig> cfgs;      // launch configurations of the per-step kernel
   int config = 0;                      // current index into cfgs
   int loop_grid = 0;                   // persistent 1D loop: blocks (0 = not available)
@@ -147,7 +148,7 @@ cudaError_t launch_step(sv_solver* s, cudaStream_t st, bool pdl = false) {
     return step1d_launch(s->p.precision, s->kp, s->buf[0], s->buf[1], s->ctl, s->ncell, s->grid, st,
                          pdl);
   return stepnd_launch(s->dim, s->p.precision, s->kp, s->buf[0], s->buf[1], s->ctl, s->g.n,
-                       c.param, st);
+                       s->nseg, st);
 }
 
 int ensure_graph(sv_solver* s) {
@@ -207,7 +208,7 @@ void build_configs(sv_solver* s) {
     }
     s->cfgs.push_back({CFG_SLIDE, 0, "1D: warps sliding over 64-cell chunks, 2 cells per thread"});
   } else {
-    const int d = stepnd_default_seg(s->dim, s->p.precision);
+    const int d = stepnd_shape(s->dim, s->p.precision).cap;
     s->cfgs.push_back({CFG_ND, d, seg_desc(d)});
     for (int seg : {64, 128, 256, 512})
       if (seg != d) s->cfgs.push_back({CFG_ND, seg, seg_desc(seg)});
@@ -223,6 +224,14 @@ int apply_config(sv_solver* s, int idx) {
     tg = tile1d_grid(s->kp, s->p.precision, c.param);
     if (tg < 1) return SV_ECUDA;
   }
+  int nseg = 1;
+  if (c.kind == CFG_ND) {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      return SV_ECUDA;
+    nseg = march_segments(stepnd_shape(s->dim, s->p.precision), s->dim, s->g.n, c.param, sms);
+  }
   if (s->graph) {
     if (cudaStreamSynchronize(s->stream) != cudaSuccess) return SV_ECUDA;
     cudaGraphExecDestroy(s->graph);
@@ -230,6 +239,7 @@ int apply_config(sv_solver* s, int idx) {
   }
   s->config = idx;
   s->tile_grid = tg;
+  s->nseg = nseg;
   return SV_OK;
 }
 

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "sv_march.h"
+
 namespace sv {
 
 struct KParams;
@@ -54,26 +56,26 @@ int heun1d_grid(const KParams& kp, int precision);
 cudaError_t heun1d_launch(int precision, int stage, const KParams& kp, void* a, void* b, Ctl* ctl,
                           int64_t N, int grid, cudaStream_t st);
 
-// 2D / 3D fused steps (sv_stepnd.cu); n[] cells per axis; seg = planes per
-// block along the marching axis (0: default)
+// 2D / 3D fused steps (sv_stepnd.cu); n[] cells per axis; nseg = segments the
+// marching axis is cut into, from march_segments (sv_march.h)
 int stepnd_grid(int dim, int precision, const KParams& kp);
-int stepnd_default_seg(int dim, int precision);
+MarchShape stepnd_shape(int dim, int precision);
 cudaError_t stepnd_launch(int dim, int precision, const KParams& kp, void* a, void* b, Ctl* ctl,
-                          const int64_t* n, int seg, cudaStream_t st);
+                          const int64_t* n, int nseg, cudaStream_t st);
 // The float 2D step marching plane pairs (sv_stepnd_pair.cu), precision
 // PREC_FP32 or PREC_FP32_PC; n == nullptr sets the kernels' shared-memory limits
-int stepnd_pair_default_seg(int dim);
+MarchShape stepnd_pair_shape();
 cudaError_t stepnd_pair_launch(int dim, int precision, const KParams& kp, void* a, void* b, Ctl* ctl,
-                               const int64_t* n, int seg, cudaStream_t st);
+                               const int64_t* n, int nseg, cudaStream_t st);
 
 // The float 3D step with the fields in packed pairs (sv_stepnd3f.cu),
 // precision PREC_FP32, PREC_FP32_PC or PREC_FP32_PS (the last compiled in
 // sv_stepnd3f_ps.cu); n == nullptr sets the kernels' shared-memory limits
-int stepnd3f_default_seg();
+MarchShape stepnd3f_shape();
 cudaError_t stepnd3f_launch(int precision, const KParams& kp, void* a, void* b, Ctl* ctl,
-                            const int64_t* n, int seg, cudaStream_t st);
+                            const int64_t* n, int nseg, cudaStream_t st);
 cudaError_t stepnd3f_launch_ps(const KParams& kp, void* a, void* b, Ctl* ctl, const int64_t* n,
-                               int seg, cudaStream_t st);
+                               int nseg, cudaStream_t st);
 
 // Batched sweep kernels of 256 (sv_batch.cu) and 128 (sv_batch128.cu) threads
 void* batch_pick256(int limiter, int precision);

@@ -417,12 +417,11 @@ template <> struct Cfg<3, PREC_FP32_P64> { static constexpr int TX = 34, TY = 15
 template <> struct Cfg<3, PREC_FP64> { static constexpr int TX = 16, TY = 16, MINB = 1, SEG = 128; };
 
 // With `n` null only the kernel's shared-memory attribute is set (done once per
-// solver at init, outside any stream capture).  `seg` = planes per block along
-// the marching axis (0: the default of Cfg); each segment pays a warm-up of
-// two planes, shorter segments give more blocks.
+// solver at init, outside any stream capture).  `nseg` = segments of the
+// marching axis (march_segments).
 template <typename R, int PP, int LIM, int SRC, int DIM, int PREC>
 static cudaError_t launch_nd(const KParams& kp, void* a, void* b, Ctl* ctl, const int64_t* n,
-                            int seg, cudaStream_t st) {
+                            int nseg, cudaStream_t st) {
   using G = Cfg<DIM, PREC>;
   constexpr size_t smem = stepnd_smem<R, DIM, G::TX, G::TY>();
   const bool bnd = DIM == 2 && (kp.bc_lo != BC_PERIODIC || kp.bc_hi != BC_PERIODIC ||
@@ -440,12 +439,7 @@ static cudaError_t launch_nd(const KParams& kp, void* a, void* b, Ctl* ctl, cons
   const int64_t nx = n[0], ny = n[1], nz = DIM == 3 ? n[2] : 1;
   const int tiles_x = (int)((nx + G::TX - 3) / (G::TX - 2));
   const int tiles_y = DIM == 3 ? (int)((ny + G::TY - 3) / (G::TY - 2)) : 1;
-  const int64_t M = DIM == 3 ? nz : ny;
-  const int64_t sl = seg > 0 ? seg : G::SEG;
-  int64_t nseg64 = (M + sl - 1) / sl;
-  if (nseg64 > M) nseg64 = M;
-  int nseg = (int)nseg64;
-  if (nseg < 1) nseg = 1;
+  if (nseg < 1 || nseg > (DIM == 3 ? nz : ny)) return cudaErrorInvalidValue;
   const int64_t blocks = (int64_t)tiles_x * tiles_y * nseg;
   if (blocks > 0x7fffffff) return cudaErrorInvalidConfiguration;
   fn<<<(int)blocks, G::TX * G::TY, smem, st>>>(kp, (R*)a, (R*)b, ctl, nx, ny, nz, tiles_x, tiles_y,
@@ -455,46 +449,50 @@ static cudaError_t launch_nd(const KParams& kp, void* a, void* b, Ctl* ctl, cons
 
 template <int LIM, int SRC, int DIM>
 static cudaError_t by_prec(int precision, const KParams& kp, void* a, void* b, Ctl* ctl,
-                           const int64_t* n, int seg, cudaStream_t st) {
+                           const int64_t* n, int nseg, cudaStream_t st) {
   switch (precision) {
-    case PREC_FP64: return launch_nd<double, 0, LIM, SRC, DIM, PREC_FP64>(kp, a, b, ctl, n, seg, st);
-    case PREC_FP32_P64: return launch_nd<float, 1, LIM, SRC, DIM, PREC_FP32_P64>(kp, a, b, ctl, n, seg, st);
+    case PREC_FP64: return launch_nd<double, 0, LIM, SRC, DIM, PREC_FP64>(kp, a, b, ctl, n, nseg, st);
+    case PREC_FP32_P64: return launch_nd<float, 1, LIM, SRC, DIM, PREC_FP32_P64>(kp, a, b, ctl, n, nseg, st);
     default:
       // the other float policies: in 2D packed plane pairs
       // (sv_stepnd_pair.cu); in 3D each cell's fields in packed pairs
       // (sv_stepnd3f.cu: plane pairs need 242 registers there, one block per
       // SM, and ran 17% slower than one cell per thread)
-      if constexpr (DIM == 2) return stepnd_pair_launch(DIM, precision, kp, a, b, ctl, n, seg, st);
-      else return stepnd3f_launch(precision, kp, a, b, ctl, n, seg, st);
+      if constexpr (DIM == 2) return stepnd_pair_launch(DIM, precision, kp, a, b, ctl, n, nseg, st);
+      else return stepnd3f_launch(precision, kp, a, b, ctl, n, nseg, st);
   }
 }
 
 template <int LIM, int DIM>
 static cudaError_t by_src(int precision, const KParams& kp, void* a, void* b, Ctl* ctl,
-                          const int64_t* n, int seg, cudaStream_t st) {
-  if (kp.frozen) return by_prec<LIM, 0, DIM>(precision, kp, a, b, ctl, n, seg, st);
-  if (kp.qi_zero) return by_prec<LIM, 1, DIM>(precision, kp, a, b, ctl, n, seg, st);
-  return by_prec<LIM, 2, DIM>(precision, kp, a, b, ctl, n, seg, st);
+                          const int64_t* n, int nseg, cudaStream_t st) {
+  if (kp.frozen) return by_prec<LIM, 0, DIM>(precision, kp, a, b, ctl, n, nseg, st);
+  if (kp.qi_zero) return by_prec<LIM, 1, DIM>(precision, kp, a, b, ctl, n, nseg, st);
+  return by_prec<LIM, 2, DIM>(precision, kp, a, b, ctl, n, nseg, st);
 }
 
 template <int DIM>
 static cudaError_t by_lim(int precision, const KParams& kp, void* a, void* b, Ctl* ctl,
-                          const int64_t* n, int seg, cudaStream_t st) {
+                          const int64_t* n, int nseg, cudaStream_t st) {
   switch (kp.limiter) {
-    case 1: return by_src<1, DIM>(precision, kp, a, b, ctl, n, seg, st);
-    case 2: return by_src<2, DIM>(precision, kp, a, b, ctl, n, seg, st);
-    default: return by_src<0, DIM>(precision, kp, a, b, ctl, n, seg, st);
+    case 1: return by_src<1, DIM>(precision, kp, a, b, ctl, n, nseg, st);
+    case 2: return by_src<2, DIM>(precision, kp, a, b, ctl, n, nseg, st);
+    default: return by_src<0, DIM>(precision, kp, a, b, ctl, n, nseg, st);
   }
 }
 
-// Default planes per block segment along the marching axis.
-int stepnd_default_seg(int dim, int precision) {
-  if ((precision == PREC_FP32 || precision == PREC_FP32_PC || precision == PREC_FP32_PS) &&
-      dim == 2)
-    return stepnd_pair_default_seg(dim);
-  if (dim == 2) return precision == PREC_FP64 ? Cfg<2, PREC_FP64>::SEG : Cfg<2, PREC_FP32_P64>::SEG;
-  if (precision == PREC_FP32_P64) return Cfg<3, PREC_FP32_P64>::SEG;
-  return precision == PREC_FP64 ? Cfg<3, PREC_FP64>::SEG : stepnd3f_default_seg();
+template <int DIM, int PREC>
+static MarchShape shape_of() {
+  using G = Cfg<DIM, PREC>;
+  return {G::TX - 2, DIM == 3 ? G::TY - 2 : 0, 1, G::MINB, {1.0, 1.75, 0.0}, G::SEG};
+}
+
+MarchShape stepnd_shape(int dim, int precision) {
+  switch (precision) {
+    case PREC_FP64: return dim == 2 ? shape_of<2, PREC_FP64>() : shape_of<3, PREC_FP64>();
+    case PREC_FP32_P64: return dim == 2 ? shape_of<2, PREC_FP32_P64>() : shape_of<3, PREC_FP32_P64>();
+    default: return dim == 2 ? stepnd_pair_shape() : stepnd3f_shape();
+  }
 }
 
 int stepnd_grid(int dim, int precision, const KParams& kp) {
@@ -505,12 +503,12 @@ int stepnd_grid(int dim, int precision, const KParams& kp) {
 }
 
 cudaError_t stepnd_launch(int dim, int precision, const KParams& kp, void* a, void* b, Ctl* ctl,
-                          const int64_t* n, int seg, cudaStream_t st) {
+                          const int64_t* n, int nseg, cudaStream_t st) {
   if (!n) return cudaErrorInvalidValue;
   int64_t ncell = n[0] * n[1] * (dim == 3 ? n[2] : 1);
   if (ncell * (dim + 3) >= (1LL << 31)) return cudaErrorInvalidValue;
-  if (dim == 2) return by_lim<2>(precision, kp, a, b, ctl, n, seg, st);
-  if (dim == 3) return by_lim<3>(precision, kp, a, b, ctl, n, seg, st);
+  if (dim == 2) return by_lim<2>(precision, kp, a, b, ctl, n, nseg, st);
+  if (dim == 3) return by_lim<3>(precision, kp, a, b, ctl, n, nseg, st);
   return cudaErrorInvalidValue;
 }
 

@@ -421,7 +421,7 @@ struct Tile3f {
 };
 
 template <int PP, int LIM, int SRC>
-cudaError_t launch3f(const KParams& kp, void* a, void* b, Ctl* ctl, const int64_t* n, int seg,
+cudaError_t launch3f(const KParams& kp, void* a, void* b, Ctl* ctl, const int64_t* n, int nseg,
                      cudaStream_t st) {
   using T = Tile3f;
   constexpr size_t smem = Lay3<T::TX, T::TY>::bytes;
@@ -430,10 +430,7 @@ cudaError_t launch3f(const KParams& kp, void* a, void* b, Ctl* ctl, const int64_
   const int64_t nx = n[0], ny = n[1], nz = n[2];
   const int tiles_x = (int)((nx + T::TX - 3) / (T::TX - 2));
   const int tiles_y = (int)((ny + T::TY - 3) / (T::TY - 2));
-  const int64_t sl = seg > 0 ? seg : T::SEG;
-  int64_t nseg64 = (nz + sl - 1) / sl;
-  if (nseg64 > nz) nseg64 = nz;
-  const int nseg = nseg64 < 1 ? 1 : (int)nseg64;
+  if (nseg < 1 || nseg > nz) return cudaErrorInvalidValue;
   const int64_t blocks = (int64_t)tiles_x * tiles_y * nseg;
   if (blocks > 0x7fffffff) return cudaErrorInvalidConfiguration;
   fn<<<(int)blocks, T::TX * T::TY, smem, st>>>(kp, (float*)a, (float*)b, ctl, nx, ny, nz, tiles_x,
@@ -442,20 +439,20 @@ cudaError_t launch3f(const KParams& kp, void* a, void* b, Ctl* ctl, const int64_
 }
 
 template <int PP, int LIM>
-cudaError_t by_src3f(const KParams& kp, void* a, void* b, Ctl* ctl, const int64_t* n, int seg,
+cudaError_t by_src3f(const KParams& kp, void* a, void* b, Ctl* ctl, const int64_t* n, int nseg,
                      cudaStream_t st) {
-  if (kp.frozen) return launch3f<PP, LIM, 0>(kp, a, b, ctl, n, seg, st);
-  if (kp.qi_zero) return launch3f<PP, LIM, 1>(kp, a, b, ctl, n, seg, st);
-  return launch3f<PP, LIM, 2>(kp, a, b, ctl, n, seg, st);
+  if (kp.frozen) return launch3f<PP, LIM, 0>(kp, a, b, ctl, n, nseg, st);
+  if (kp.qi_zero) return launch3f<PP, LIM, 1>(kp, a, b, ctl, n, nseg, st);
+  return launch3f<PP, LIM, 2>(kp, a, b, ctl, n, nseg, st);
 }
 
 template <int PP>
-cudaError_t by_lim3f(const KParams& kp, void* a, void* b, Ctl* ctl, const int64_t* n, int seg,
+cudaError_t by_lim3f(const KParams& kp, void* a, void* b, Ctl* ctl, const int64_t* n, int nseg,
                      cudaStream_t st) {
   switch (kp.limiter) {
-    case 1: return by_src3f<PP, 1>(kp, a, b, ctl, n, seg, st);
-    case 2: return by_src3f<PP, 2>(kp, a, b, ctl, n, seg, st);
-    default: return by_src3f<PP, 0>(kp, a, b, ctl, n, seg, st);
+    case 1: return by_src3f<PP, 1>(kp, a, b, ctl, n, nseg, st);
+    case 2: return by_src3f<PP, 2>(kp, a, b, ctl, n, nseg, st);
+    default: return by_src3f<PP, 0>(kp, a, b, ctl, n, nseg, st);
   }
 }
 

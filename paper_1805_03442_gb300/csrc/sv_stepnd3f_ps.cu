@@ -5,8 +5,8 @@
 namespace sv {
 
 cudaError_t stepnd3f_launch_ps(const KParams& kp, void* a, void* b, Ctl* ctl, const int64_t* n,
-                               int seg, cudaStream_t st) {
-  return by_lim3f<3>(kp, a, b, ctl, n, seg, st);
+                               int nseg, cudaStream_t st) {
+  return by_lim3f<3>(kp, a, b, ctl, n, nseg, st);
 }
 
 }  // namespace sv

@@ -422,10 +422,10 @@ stepnd_pair_kernel(const KParams kp, float* __restrict__ bufA, float* __restrict
 // Tiles of the pair kernel: 128 threads along x (126 interior cells), 166-168
 // registers, 3 blocks per SM (a budget of 4 spills).
 template <int DIM> struct PairCfg;
-template <> struct PairCfg<2> { static constexpr int TX = 128, TY = 1, MINB = 3, SEG = 128; };
+template <> struct PairCfg<2> { static constexpr int TX = 128, TY = 1, MINB = 3, SEG = 256; };
 
 template <int PP, int LIM, int SRC, int DIM>
-cudaError_t launch_pair(const KParams& kp, void* a, void* b, Ctl* ctl, const int64_t* n, int seg,
+cudaError_t launch_pair(const KParams& kp, void* a, void* b, Ctl* ctl, const int64_t* n, int nseg,
                         cudaStream_t st) {
   using G = PairCfg<DIM>;
   constexpr size_t smem = pair_smem<DIM, G::TX, G::TY>();
@@ -444,11 +444,7 @@ cudaError_t launch_pair(const KParams& kp, void* a, void* b, Ctl* ctl, const int
   const int64_t nx = n[0], ny = n[1], nz = DIM == 3 ? n[2] : 1;
   const int tiles_x = (int)((nx + G::TX - 3) / (G::TX - 2));
   const int tiles_y = DIM == 3 ? (int)((ny + G::TY - 3) / (G::TY - 2)) : 1;
-  const int64_t M = DIM == 3 ? nz : ny;
-  const int64_t sl = seg > 0 ? seg : G::SEG;
-  int64_t nseg64 = (M + sl - 1) / sl;
-  if (nseg64 > M) nseg64 = M;
-  const int nseg = (int)nseg64;
+  if (nseg < 1 || nseg > (DIM == 3 ? nz : ny)) return cudaErrorInvalidValue;
   const int64_t blocks = (int64_t)tiles_x * tiles_y * nseg;
   if (blocks > 0x7fffffff) return cudaErrorInvalidConfiguration;
   fn<<<(int)blocks, G::TX * G::TY, smem, st>>>(kp, (float*)a, (float*)b, ctl, nx, ny, nz, tiles_x,
@@ -457,14 +453,14 @@ cudaError_t launch_pair(const KParams& kp, void* a, void* b, Ctl* ctl, const int
 }
 
 template <int PP, int DIM>
-cudaError_t pair_by_kind(const KParams& kp, void* a, void* b, Ctl* ctl, const int64_t* n, int seg,
+cudaError_t pair_by_kind(const KParams& kp, void* a, void* b, Ctl* ctl, const int64_t* n, int nseg,
                          cudaStream_t st) {
   const int src = kp.frozen ? 0 : (kp.qi_zero ? 1 : 2);
 #define SV_PAIR_SRC(LIM)                                                   \
   switch (src) {                                                           \
-    case 0: return launch_pair<PP, LIM, 0, DIM>(kp, a, b, ctl, n, seg, st);    \
-    case 1: return launch_pair<PP, LIM, 1, DIM>(kp, a, b, ctl, n, seg, st);    \
-    default: return launch_pair<PP, LIM, 2, DIM>(kp, a, b, ctl, n, seg, st);   \
+    case 0: return launch_pair<PP, LIM, 0, DIM>(kp, a, b, ctl, n, nseg, st);    \
+    case 1: return launch_pair<PP, LIM, 1, DIM>(kp, a, b, ctl, n, nseg, st);    \
+    default: return launch_pair<PP, LIM, 2, DIM>(kp, a, b, ctl, n, nseg, st);   \
   }
   switch (kp.limiter) {
     case 1: SV_PAIR_SRC(1)
@@ -476,18 +472,23 @@ cudaError_t pair_by_kind(const KParams& kp, void* a, void* b, Ctl* ctl, const in
 
 }  // namespace
 
-int stepnd_pair_default_seg(int) { return PairCfg<2>::SEG; }
+// An iteration of one, two or three blocks on an SM: 1.2, 1.6 and 2.4 us
+// (1000 x 700 cells), the issue slots being shared beyond one block.
+MarchShape stepnd_pair_shape() {
+  using G = PairCfg<2>;
+  return {G::TX - 2, 0, 2, G::MINB, {1.0, 1.3, 2.0}, G::SEG};
+}
 
 // n == nullptr: set the kernels' shared-memory limits (host side, at set-up).
 // 2D only: in 3D the pair kernel needs 242 registers (one 8-warp block per SM)
 // and loses to one cell per thread.
 cudaError_t stepnd_pair_launch(int dim, int precision, const KParams& kp, void* a, void* b, Ctl* ctl,
-                               const int64_t* n, int seg, cudaStream_t st) {
+                               const int64_t* n, int nseg, cudaStream_t st) {
   if (dim == 2)
     switch (precision) {
-      case PREC_FP32_PC: return pair_by_kind<2, 2>(kp, a, b, ctl, n, seg, st);
-      case PREC_FP32_PS: return pair_by_kind<3, 2>(kp, a, b, ctl, n, seg, st);
-      default: return pair_by_kind<0, 2>(kp, a, b, ctl, n, seg, st);
+      case PREC_FP32_PC: return pair_by_kind<2, 2>(kp, a, b, ctl, n, nseg, st);
+      case PREC_FP32_PS: return pair_by_kind<3, 2>(kp, a, b, ctl, n, nseg, st);
+      default: return pair_by_kind<0, 2>(kp, a, b, ctl, n, nseg, st);
     }
   return cudaErrorInvalidValue;
 }
