@@ -69,11 +69,13 @@ extern "C" {
 /* ---- arithmetic of the step kernels */
 #define SV_FP32     0   /* float state and arithmetic */
 #define SV_FP64     1   /* double state and arithmetic */
-#define SV_FP32_P64 2   /* float state, pressure recovery of eq. 5 in double */
-#define SV_FP32_PC  3   /* float state, pressure recovery of eq. 5 in compensated float:
-                           the exact E - rho v^2/2 - E_nu of the float operands (two
-                           error-free float sums), times gamma - 1, rounded once; the
-                           same p as SV_FP32_P64 to within its last bit, at float speed */
+#define SV_FP32_P64 2   /* float state, pressure recovery of eq. 5 to double accuracy: the
+                           exact E - rho v^2/2 - E_nu of the float operands, times
+                           gamma - 1 held to ~2^-48, rounded once (within the last bit of
+                           the subtraction carried out in double) */
+#define SV_FP32_PC  3   /* the same arithmetic (two error-free float sums) under the name of
+                           the compensated-float policy, with that policy's choice of
+                           launch configurations */
 #define SV_FP32_PS  4   /* MUSCL-Hancock (1D, 2D, 3D): float perturbations about the uniform
                            equilibrium (rho = p = 1, v = 0, E_nu = C_k + S) on the device, the
                            fluxes and the source Y written so that the equilibrium part cancels

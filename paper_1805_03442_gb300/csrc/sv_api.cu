@@ -206,7 +206,12 @@ void build_configs(sv_solver* s) {
       s->cfgs.push_back({CFG_TILE, 14,
                          "1D: 512-cell block tiles, 2 cells per thread, 64 registers, 4 blocks/SM"});
     }
-    s->cfgs.push_back({CFG_SLIDE, 0, "1D: warps sliding over 64-cell chunks, 2 cells per thread"});
+    if (s->p.precision == SV_FP32_P64 && s->p.method == SV_HANCOCK && s->ncell >= kTile1dMinCells)
+      // one configuration: the float policies' default one
+      s->cfgs.push_back({CFG_TILE, 13,
+                         "1D: 512-cell block tiles, 2 cells per thread, 78 registers, 3 blocks/SM"});
+    else
+      s->cfgs.push_back({CFG_SLIDE, 0, "1D: warps sliding over 64-cell chunks, 2 cells per thread"});
   } else {
     const int d = stepnd_shape(s->dim, s->p.precision).cap;
     s->cfgs.push_back({CFG_ND, d, seg_desc(d)});

@@ -230,7 +230,7 @@ template <int NTB, int LIM>
 void* bpick_prec(int precision) {
   switch (precision) {
     case PREC_FP64: return (void*)KB<NTB, double, 0, LIM>::fn;
-    case PREC_FP32_P64: return (void*)KB<NTB, float, 1, LIM>::fn;
+    case PREC_FP32_P64:
     case PREC_FP32_PC: return (void*)KB<NTB, float, 2, LIM>::fn;
     case PREC_FP32_PS: return (void*)KB<NTB, float, 3, LIM>::fn;
     default: return (void*)KB<NTB, float, 0, LIM>::fn;

@@ -286,21 +286,21 @@ template <> struct StepDt<float> {
 
 // ---------------------------------------------------------------- eq. 5
 
-// Pressure policies of the float kernels: PP = 0 all-float, PP = 1 the
-// subtraction of eq. 5 carried out in double, PP = 2 the same subtraction in
-// compensated float: E - kin2/2 - E_nu of the float operands is formed exactly
-// as an unevaluated sum t + e by two of Dekker's fast two-sums (exact when
-// |E| >= E_nu and E - E_nu >= kin2/2, i.e. for every state with p >= 0), then
-// multiplied by g1 held as two floats (g1 + g1lo) with one final rounding.  The
-// result is the double policy's p to within its last bit, at the cost of eleven
-// float operations (three for PP = 0) instead of a trip through GB300's narrow
-// FP64 pipe.
+// Pressure policies of the float kernels: PP = 0 all-float, PP = 2 the
+// subtraction of eq. 5 without rounding: E - kin2/2 - E_nu of the float operands
+// is formed exactly as an unevaluated sum t + e by two of Dekker's fast two-sums
+// (exact when |E| >= E_nu and E - E_nu >= kin2/2, i.e. for every state with
+// p >= 0; the sign of p is right for every state), then multiplied by g1 held as
+// two floats (g1 + g1lo) with one final rounding.  It serves both SV_FP32_PC and
+// SV_FP32_P64: the subtraction carried out in double gives the same p to within
+// its last bit (tests/test_pressure_split.py), but GB300's FP64 pipe (two lanes
+// per SM) makes each of its four conversions and three operations cost 16 cycles
+// of an SM for 32 cells.  Measured in double / this way, per step: 1D 2^22 412 /
+// 54 us, 3D 201 x 150 x 170 1660 / 345 us.
 template <typename R, int PP>
 __device__ __forceinline__ R pressure(const P<R>& k, R kin2, R E, R Ev) {
   // kin2 = rho |v|^2 (twice the kinetic energy density)
-  if constexpr (PP == 1) {
-    return (R)((double)k.g1 * ((double)E - 0.5 * (double)kin2 - (double)Ev));
-  } else if constexpr (PP == 2) {
+  if constexpr (PP == 2) {
     static_assert(std::is_same<R, float>::value, "compensated pressure is a float policy");
     const float h = 0.5f * kin2;
     const float s = __fsub_rn(E, Ev);

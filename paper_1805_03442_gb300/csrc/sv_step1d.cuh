@@ -302,11 +302,8 @@ __device__ __forceinline__ void step1d_warp(const P<R>& k, const R* __restrict__
   const int src_m = (lane + 31) & 31, src_p = (lane + 1) & 31;
   // The float MUSCL-Hancock step (float or compensated-float pressure, or the
   // perturbation layout) runs both cells of a lane in packed f32x2 arithmetic
-  // (sv_pair1d.cuh, sv_pert1d.cuh); double, double-pressure and Heun stay
-  // scalar.
-  constexpr bool PACKED = std::is_same<R, float>::value && (PP == 0 || PP == 2 || PP == 3) &&
-                          MODE == MODE_HANCOCK;
-  constexpr int PPK = PP == 1 ? 0 : PP;     // the packed policy (unused when not PACKED)
+  // (sv_pair1d.cuh, sv_pert1d.cuh); double and Heun stay scalar.
+  constexpr bool PACKED = std::is_same<R, float>::value && MODE == MODE_HANCOCK;
   using pk::f2;
   // carried from chunk to chunk: the odd cell's right face state (its first
   // use, by lane 0 of the warm-up chunk, only needs to be physical), the
@@ -338,10 +335,10 @@ __device__ __forceinline__ void step1d_warp(const P<R>& k, const R* __restrict__
         B[f] = pk::pair(c, rf[(pos + 2) & MASK] - X[f].y);
       }
       f2 WP[4], WM[4], YE, YEv, L[4], F[4];
-      pkx::predict<PPK, LIM, SRC>(k, X, A, B, ndt_2h2, dt_22, WP, WM, YE, YEv);
+      pkx::predict<PP, LIM, SRC>(k, X, A, B, ndt_2h2, dt_22, WP, WM, YE, YEv);
 #pragma unroll
       for (int f = 0; f < 4; ++f) L[f] = pk::pair(shfl(lane == 31 ? Wy_prev[f] : WP[f].y, src_m), WP[f].x);
-      pkx::hll<PPK>(k, L, WM, xl, X, F);            // faces 2i - 1/2 and 2i + 1/2
+      pkx::hll<PP>(k, L, WM, xl, X, F);            // faces 2i - 1/2 and 2i + 1/2
       if (kk > c0) {
         // update of the pair of chunk kk-1: left faces F_prev, right faces
         // (inner face, next lane's left face)
@@ -354,7 +351,7 @@ __device__ __forceinline__ void step1d_warp(const P<R>& k, const R* __restrict__
           f2 Nw[4];
           pk::update<SRC>(Qp, F_prev, FRt, YE_prev, YEv_prev, dt2, ndtdx2, Nw);
           const bool two = jo + 1 < N;
-          pkx::cfl<PPK, SRC>(k, Nw, two ? 3 : 1, smax, akey, flags);
+          pkx::cfl<PP, SRC>(k, Nw, two ? 3 : 1, smax, akey, flags);
           if (two && (stride % 2) == 0) {
 #pragma unroll
             for (int f = 0; f < 4; ++f) *reinterpret_cast<f2*>(Uout + f * stride + jo) = Nw[f];

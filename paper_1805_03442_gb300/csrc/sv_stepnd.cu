@@ -411,9 +411,7 @@ stepnd_kernel(const KParams kp, R* __restrict__ bufA, R* __restrict__ bufB, Ctl*
 // ------------------------------------------------------------------ launch
 
 template <int DIM, int PREC> struct Cfg;
-template <> struct Cfg<2, PREC_FP32_P64> { static constexpr int TX = 256, TY = 1, MINB = 2, SEG = 256; };
 template <> struct Cfg<2, PREC_FP64> { static constexpr int TX = 128, TY = 1, MINB = 2, SEG = 256; };
-template <> struct Cfg<3, PREC_FP32_P64> { static constexpr int TX = 34, TY = 15, MINB = 1, SEG = 128; };
 template <> struct Cfg<3, PREC_FP64> { static constexpr int TX = 16, TY = 16, MINB = 1, SEG = 128; };
 
 // With `n` null only the kernel's shared-memory attribute is set (done once per
@@ -452,9 +450,8 @@ static cudaError_t by_prec(int precision, const KParams& kp, void* a, void* b, C
                            const int64_t* n, int nseg, cudaStream_t st) {
   switch (precision) {
     case PREC_FP64: return launch_nd<double, 0, LIM, SRC, DIM, PREC_FP64>(kp, a, b, ctl, n, nseg, st);
-    case PREC_FP32_P64: return launch_nd<float, 1, LIM, SRC, DIM, PREC_FP32_P64>(kp, a, b, ctl, n, nseg, st);
     default:
-      // the other float policies: in 2D packed plane pairs
+      // the float policies: in 2D packed plane pairs
       // (sv_stepnd_pair.cu); in 3D each cell's fields in packed pairs
       // (sv_stepnd3f.cu: plane pairs need 242 registers there, one block per
       // SM, and ran 17% slower than one cell per thread)
@@ -490,7 +487,6 @@ static MarchShape shape_of() {
 MarchShape stepnd_shape(int dim, int precision) {
   switch (precision) {
     case PREC_FP64: return dim == 2 ? shape_of<2, PREC_FP64>() : shape_of<3, PREC_FP64>();
-    case PREC_FP32_P64: return dim == 2 ? shape_of<2, PREC_FP32_P64>() : shape_of<3, PREC_FP32_P64>();
     default: return dim == 2 ? stepnd_pair_shape() : stepnd3f_shape();
   }
 }

@@ -15,7 +15,7 @@ MarchShape stepnd3f_shape() {
 cudaError_t stepnd3f_launch(int precision, const KParams& kp, void* a, void* b, Ctl* ctl,
                             const int64_t* n, int nseg, cudaStream_t st) {
   if (precision == PREC_FP32_PS) return stepnd3f_launch_ps(kp, a, b, ctl, n, nseg, st);
-  if (precision == PREC_FP32_PC) return by_lim3f<2>(kp, a, b, ctl, n, nseg, st);
+  if (precision == PREC_FP32_PC || precision == PREC_FP32_P64) return by_lim3f<2>(kp, a, b, ctl, n, nseg, st);
   if (precision == PREC_FP32) return by_lim3f<0>(kp, a, b, ctl, n, nseg, st);
   return cudaErrorInvalidValue;
 }

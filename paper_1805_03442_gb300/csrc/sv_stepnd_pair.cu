@@ -486,6 +486,7 @@ cudaError_t stepnd_pair_launch(int dim, int precision, const KParams& kp, void* 
                                const int64_t* n, int nseg, cudaStream_t st) {
   if (dim == 2)
     switch (precision) {
+      case PREC_FP32_P64:
       case PREC_FP32_PC: return pair_by_kind<2, 2>(kp, a, b, ctl, n, nseg, st);
       case PREC_FP32_PS: return pair_by_kind<3, 2>(kp, a, b, ctl, n, nseg, st);
       default: return pair_by_kind<0, 2>(kp, a, b, ctl, n, nseg, st);

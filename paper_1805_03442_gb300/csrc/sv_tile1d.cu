@@ -7,7 +7,7 @@ namespace sv {
 namespace {
 
 void* pick(const KParams& kp, int precision, int var) {
-  if (precision == PREC_FP32_PC) return tile1d_pick_pc(kp, var);
+  if (precision == PREC_FP32_PC || precision == PREC_FP32_P64) return tile1d_pick_pc(kp, var);
   if (precision == PREC_FP32_PS) return tile1d_pick_ps(kp, var);
   return pick_lim<0>(kp, var);
 }

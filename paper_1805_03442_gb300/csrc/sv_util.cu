@@ -118,9 +118,6 @@ cudaError_t dt_reduce_launch(int precision, int dim, const KParams& kp, const vo
                                                      dim, ncell);
       break;
     case PREC_FP32_P64:
-      dt_reduce_kernel<float, 1><<<g, NTU, 0, st>>>(kp, (const float*)a, (const float*)b, ctl,
-                                                    dim, ncell);
-      break;
     case PREC_FP32_PC:
       dt_reduce_kernel<float, 2><<<g, NTU, 0, st>>>(kp, (const float*)a, (const float*)b, ctl,
                                                     dim, ncell);
