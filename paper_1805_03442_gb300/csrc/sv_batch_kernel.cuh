@@ -78,13 +78,17 @@ batch_kernel(RunDev* __restrict__ runs, const int* __restrict__ order, int nruns
   __shared__ uint32_t s_f[NTB / 32];
   __shared__ int s_run, s_stop, s_last, s_log;
   __shared__ double s_dt, s_t;
+  __shared__ float s_word;              // speed threshold of the double bound (d64::Bound)
   __shared__ R s_step[4];               // dt, dt/h, dt/(2h), dt/2 of the next step
   extern __shared__ __align__(16) unsigned char smemb[];   // per-warp rings
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   R* ring = reinterpret_cast<R*>(smemb) + warp * (ring1d_bytes<R>() / sizeof(R));
 
   for (;;) {
-    if (threadIdx.x == 0) s_run = atomicAdd(queue, 1);
+    if (threadIdx.x == 0) {
+      s_run = atomicAdd(queue, 1);
+      s_word = 0.0f;
+    }
     __syncthreads();
     const int qi = s_run;
     if (qi >= nruns) break;
@@ -123,15 +127,16 @@ batch_kernel(RunDev* __restrict__ runs, const int* __restrict__ order, int nruns
 
     // dt of the initial state (same per-cell bound as every step)
     {
-      R smax = 0, akey = -INFINITY;
-      uint32_t flags = 0;
+      Acc<R> acc(&s_word);
       for (int j = threadIdx.x; j < n; j += NTB) {
         const R u[4] = {A[j], A[stride + j], A[2 * stride + j], A[3 * stride + j]};
-        cell_bound<R, PP, 1>(k, u, smax, akey, flags);
+        cell_bound<PP, 1>(k, u, acc);
       }
-      block_max<NTB>(smax, akey, flags, s_a, s_b, s_f);
+      block_max<NTB>(acc.smax, acc.akey, acc.flags, s_a, s_b, s_f);
       if (threadIdx.x == 0) {
-        const double dt = dt_from_maxima(kp, smax, akey, flags);
+        s_word = 0.0f;
+        uint32_t flags = acc.flags;
+        const double dt = dt_from_maxima(kp, acc.smax, acc.akey, flags);
         double t = rd->t;
         rd->flags = flags;
         s_t = t;
@@ -164,24 +169,25 @@ batch_kernel(RunDev* __restrict__ runs, const int* __restrict__ order, int nruns
       const R dt = s_step[0], dtdx = s_step[1], dt_2h = s_step[2], dt_2 = s_step[3];
       const R* Uin = cur ? B : A;
       R* Uout = cur ? A : B;
-      R smax = 0, akey = -INFINITY;
-      uint32_t flags = 0;
+      Acc<R> acc(&s_word);
       if (src == 0)
         step1d_warp<R, PP, LIM, 0>(k, Uin, Uout, n, stride, c0, c1, lane, dt, dtdx, dt_2h, dt_2,
-                                   smax, akey, flags, ring, kp, s_t);
+                                   acc, ring, kp, s_t);
       else if (src == 1)
         step1d_warp<R, PP, LIM, 1>(k, Uin, Uout, n, stride, c0, c1, lane, dt, dtdx, dt_2h, dt_2,
-                                   smax, akey, flags, ring, kp, s_t);
+                                   acc, ring, kp, s_t);
       else
         step1d_warp<R, PP, LIM, 2>(k, Uin, Uout, n, stride, c0, c1, lane, dt, dtdx, dt_2h, dt_2,
-                                   smax, akey, flags, ring, kp, s_t);
+                                   acc, ring, kp, s_t);
       // the barrier inside block_max also orders this step's stores before the
       // next step's loads of neighbouring warps' cells
-      block_max<NTB>(smax, akey, flags, s_a, s_b, s_f);
+      block_max<NTB>(acc.smax, acc.akey, acc.flags, s_a, s_b, s_f);
       cur ^= 1u;
       ++steps;
       if (threadIdx.x == 0) {
-        const double dt_next = dt_from_maxima(kp, smax, akey, flags);
+        s_word = 0.0f;
+        uint32_t flags = acc.flags;
+        const double dt_next = dt_from_maxima(kp, acc.smax, acc.akey, flags);
         const double t = s_last ? t_end : s_t + dtd;
         s_t = t;
         if (steps >= max_steps && t < t_end) flags |= FLAG_MAXSTEPS;

@@ -35,12 +35,11 @@ heun1d_kernel(const KParams kp, R* __restrict__ bufA, R* __restrict__ bufB, Ctl*
   const int nchunk = (N + 63) / 64;
   const int c0 = (int)((int64_t)warp * nchunk / nwarps);
   const int c1 = (int)((int64_t)(warp + 1) * nchunk / nwarps);
-  R smax = 0, akey = -INFINITY;
-  uint32_t flags = 0;
+  Acc<R> acc(bound_word());
   step1d_warp<R, PP, LIM, SRC, MODE>(k, Uin, Uout, N, N, c0, c1, lane, sd.dt, sd.dtdx, sd.dt_2h,
-                                     sd.dt_2, smax, akey, flags, ring, kp, sc.t, Un);
+                                     sd.dt_2, acc, ring, kp, sc.t, Un);
   if (MODE == MODE_HEUN2)
-    reduce_and_finalize<R, NTH>(ctl, kp, smax, akey, flags, true, false);
+    reduce_and_finalize<R, NTH>(ctl, kp, acc.smax, acc.akey, acc.flags, true, false);
 }
 
 template <typename R, int LIM, int SRC, int MODE>

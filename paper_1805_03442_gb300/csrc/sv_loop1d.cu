@@ -85,11 +85,10 @@ loop1d_kernel(const KParams kp, R* bufA, R* bufB, Ctl* ctl, int N, long long nma
     const R* Uin = sc.cur ? bufB : bufA;
     R* Uout = sc.cur ? bufA : bufB;
     const StepDt<R> sd(sc);
-    R smax = 0, akey = -INFINITY;
-    uint32_t flags = 0;
+    Acc<R> acc(bound_word());
     step1d_warp<R, PP, LIM, SRC>(k, Uin, Uout, N, N, c0, c1, lane, sd.dt, sd.dtdx, sd.dt_2h,
-                                 sd.dt_2, smax, akey, flags, ring, kp, sc.t);
-    const bool last = block_arrive<NTL, R>(ctl, smax, akey, flags);
+                                 sd.dt_2, acc, ring, kp, sc.t);
+    const bool last = block_arrive<NTL, R>(ctl, acc.smax, acc.akey, acc.flags);
     if (threadIdx.x == 0) {
       bool ok = true;
       if (last) {

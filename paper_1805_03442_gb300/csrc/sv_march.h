@@ -1,8 +1,8 @@
 // sv_march.h -- how many segments the marching axis of a 2D / 3D step is cut
 // into (host only).
 //
-// A block marches over one segment of one transverse tile and pays two extra
-// iterations of warm-up, so few long segments do the least work; but a grid
+// A block marches over one segment of one transverse tile and pays up to two
+// extra iterations of warm-up, so few long segments do the least work; but a grid
 // of few tiles needs many segments to reach every SM, and a grid of many
 // needs a count whose last wave of blocks is not nearly empty.  The rule
 // minimises
@@ -29,6 +29,7 @@ namespace sv {
 struct MarchShape {
   int cols_x, cols_y;     // written columns of a tile (cols_y 0: 2D)
   int step;               // planes an iteration takes (the row pairs: 2)
+  double warm;            // a segment's extra iterations, in whole ones
   int occ;                // blocks per SM
   double t[3];            // t[k - 1]: iteration time with k blocks on the SM
   int cap;                // default cap on a segment's planes
@@ -50,7 +51,7 @@ inline int march_segments(const MarchShape& g, int dim, const int64_t* n, int64_
   double best_cost = 1e300;
   for (int64_t s = best; s <= hi; ++s) {
     const int64_t planes = (M + s - 1) / s;
-    const double iters = (double)((planes + g.step - 1) / g.step + 2);
+    const double iters = (double)((planes + g.step - 1) / g.step) + g.warm;
     const int64_t blocks = tiles * s, slots = (int64_t)sms * g.occ;
     const int64_t full = blocks / slots, rem = blocks % slots;
     double cost = (double)full * g.t[g.occ - 1] * iters;

@@ -9,9 +9,8 @@
 //   F/G of eq. 15                  (rho v_a, rho v v_a + p e_a, v_a (E + p), v_a E_nu)
 //   eq. 13                         HLL flux with Davis speed estimates
 //
-// Everything is templated on the arithmetic type R (float or double).  The
-// float instantiation uses the SFU approximations (rcp, rsqrt, lg2, ex2); the
-// double instantiation uses IEEE division, sqrt and pow.
+// The float kernels use the SFU approximations (rcp, rsqrt, lg2, ex2); the
+// arithmetic of the double kernels is in sv_f64.cuh.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -59,6 +58,10 @@ struct KParams {
   double S;
   double ref[4];
   float fps[4];
+  // for the double kernels' bound (sv_f64.cuh): log2(gamma - 1), log2 of
+  // cfl h / (c_tau tau0) (the tau / tau0 at which the tau cap meets a unit
+  // signal speed), and the margin its float estimate of log2(tau / tau0) keeps
+  float fb[4];
 };
 
 // Fill the float copies once on the host, so float kernels convert nothing.
@@ -83,6 +86,10 @@ inline void kparams_finish(KParams& k) {
   k.fps[1] = (float)ev0;
   k.fps[2] = (float)k.S;
   k.fps[3] = 0.0f;
+  k.fb[0] = (float)log2(k.g1);
+  k.fb[1] = k.frozen ? 0.0f : (float)log2(k.cfl * k.h / (k.c_tau * k.tau0));
+  k.fb[2] = (float)(1e-4 * (1.0 + fabs(k.tau_rho) + fabs(k.tau_T)));
+  k.fb[3] = 0.0f;
 }
 
 // Entry f of the perturbation layout's reference state U_ref for nf = DIM + 3
@@ -163,29 +170,15 @@ template <> struct Ar<float> {
   }
 };
 
-// The double kernels' reciprocal: the SFU's approximate 1/x refined by two
-// Newton-Raphson steps y <- y + y (1 - x y) (each doubling the correct bits;
-// within an ulp or two of 1/x for the positive normal densities and speed sums
-// it is used on): four FMAs instead of an IEEE division on GB300's narrow FP64
-// pipe.  A non-positive density still raises SV_FLAG_NONPHYS through the
-// physicality checks, which test rho itself.
-template <> struct Ar<double> {
-  static __device__ __forceinline__ double rcp(double x) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    y = fma(y, fma(-x, y, 1.0), y);
-    return fma(y, fma(-x, y, 1.0), y);
-  }
-  static __device__ __forceinline__ double sqrt_pos(double x) { return sqrt(x); }
-};
 
 // Parameters converted once to the kernel's arithmetic type.
 template <typename R> struct P;
 
 template <> struct P<double> {
-  double gamma, g1, Ck, Q0, inv_tau0, tau0;
+  double g1, gg1, Ck, Q0, inv_tau0, tau0;   // gg1 = gamma (gamma - 1)
   double tau_rho, tau_T, Q_rho, Q_T, I_rho, I_T;
-  int limiter, frozen, qi_zero, bc_lo, bc_hi;
+  float lg_g1, l0, l_margin, f_tau_rho, f_tau_T;   // the bound's float estimates
+  int bc_lo, bc_hi;
   // eq. 6 exponents that are multiples of 1/2 (the paper's tau_rho = -1,
   // tau_T = -1.5): twice each exponent (tau_rho, tau_T, Q_rho, Q_T, I_rho,
   // I_T), and whether the tau pair / the Q and I exponents all qualify
@@ -193,10 +186,10 @@ template <> struct P<double> {
   int hk[6];
   bool half_tau, half_qi;
   __device__ __forceinline__ explicit P(const KParams& k)
-      : gamma(k.gamma), g1(k.g1), Ck(k.Ck), Q0(k.Q0), inv_tau0(k.inv_tau0), tau0(k.tau0),
+      : g1(k.g1), gg1(k.gamma * k.g1), Ck(k.Ck), Q0(k.Q0), inv_tau0(k.inv_tau0), tau0(k.tau0),
         tau_rho(k.tau_rho), tau_T(k.tau_T), Q_rho(k.Q_rho), Q_T(k.Q_T), I_rho(k.I_rho),
-        I_T(k.I_T), limiter(k.limiter), frozen(k.frozen), qi_zero(k.qi_zero), bc_lo(k.bc_lo),
-        bc_hi(k.bc_hi) {
+        I_T(k.I_T), lg_g1(k.fb[0]), l0(k.fb[1]), l_margin(k.fb[2]), f_tau_rho(k.f[6]),
+        f_tau_T(k.f[7]), bc_lo(k.bc_lo), bc_hi(k.bc_hi) {
     const double e[6] = {tau_rho, tau_T, Q_rho, Q_T, I_rho, I_T};
     bool ok[6];
 #pragma unroll
@@ -209,13 +202,6 @@ template <> struct P<double> {
     half_qi = ok[2] && ok[3] && ok[4] && ok[5];
   }
 };
-
-// rho^(kr/2) T^(kT/2) for integers |kr|, |kT| <= 8, given sr = sqrt(rho) and
-// sT = sqrt(T) where kr / kT is odd: whole powers by repeated multiplication,
-// the negative ones gathered into one reciprocal.  Each product rounds once,
-// so the result stays within a few ulp of pow's.
-__device__ __forceinline__ double half_powers(double rho, double sr, int kr, double T, double sT,
-                                              int kT);
 
 template <> struct P<float> {
   float gamma, g1, Ck, Q0, inv_tau0, tau0;
@@ -244,10 +230,17 @@ struct StepCtl {
   uint32_t cur, gen;
 };
 
+// The block's shared word of the double bound's speed threshold (d64::Bound).
+__device__ __forceinline__ float* bound_word() {
+  __shared__ float s_word;
+  return &s_word;
+}
+
 // Must be called by every thread of the block; ends with a block barrier.
 __device__ __forceinline__ StepCtl block_step_ctl(const Ctl* ctl) {
   __shared__ StepCtl s;
   if (threadIdx.x == 0) {
+    *bound_word() = 0.0f;
     const volatile Ctl* c = (const volatile Ctl*)ctl;
     s.t = c->t;
     s.dt = c->dt;
@@ -297,25 +290,22 @@ template <> struct StepDt<float> {
 // per SM) makes each of its four conversions and three operations cost 16 cycles
 // of an SM for 32 cells.  Measured in double / this way, per step: 1D 2^22 412 /
 // 54 us, 3D 201 x 150 x 170 1660 / 345 us.
-template <typename R, int PP>
-__device__ __forceinline__ R pressure(const P<R>& k, R kin2, R E, R Ev) {
+template <int PP>
+__device__ __forceinline__ float pressure(const P<float>& k, float kin2, float E, float Ev) {
   // kin2 = rho |v|^2 (twice the kinetic energy density)
   if constexpr (PP == 2) {
-    static_assert(std::is_same<R, float>::value, "compensated pressure is a float policy");
     const float h = 0.5f * kin2;
     const float s = __fsub_rn(E, Ev);
     const float e1 = __fsub_rn(__fsub_rn(E, s), Ev);
     const float t = __fsub_rn(s, h);
     const float e2 = __fsub_rn(__fsub_rn(s, t), h);
     return __fmaf_rn(k.g1, t, __fmaf_rn(k.g1lo, t, __fmul_rn(k.g1, __fadd_rn(e1, e2))));
-  } else if constexpr (std::is_same<R, float>::value) {
+  } else {
     // The cancelling pair first: E - E_nu is exact whenever E_nu >= E / 2
     // (Sterbenz), which is where the cancellation bites, so p stays within
     // ~1.4 ulp of the exact value of the float operands however large E_nu
     // is (the order E - kin2/2 - E_nu loses log2(E / p) bits there).
     return k.g1 * fmaf(kin2, -0.5f, E - Ev);
-  } else {
-    return k.g1 * (E - (R)0.5 * kin2 - Ev);
   }
 }
 
@@ -361,21 +351,21 @@ __device__ __forceinline__ bool both_positive(double a, double b) {
 
 // TVD slope limiters on the two one-sided differences a, b (eq. 14 asks for
 // "limiter functions" without naming one): LIM 0 minmod, 1 van Leer, 2 MC.
-template <int LIM, typename R>
-__device__ __forceinline__ R limit(R a, R b) {
+// (Double: d64::limit of sv_f64.cuh.)
+template <int LIM>
+__device__ __forceinline__ float limit(float a, float b) {
   if constexpr (LIM == 0) {
     return minmod(a, b);
   } else {
-    const R ab = a * b;
-    R m;
+    const float ab = a * b;
+    float m;
     if (LIM == 1) {
-      if constexpr (std::is_same<R, float>::value) m = __fdividef(2.0f * ab, fabsf(a + b));
-      else m = (R)2 * ab / fabs(a + b);
+      m = __fdividef(2.0f * ab, fabsf(a + b));
     } else {
-      m = fmin(fabs(a), fabs(b));
-      m = fmin((R)2 * m, (R)0.5 * fabs(a + b));
+      m = fminf(fabsf(a), fabsf(b));
+      m = fminf(2.0f * m, 0.5f * fabsf(a + b));
     }
-    return ab > (R)0 ? copysign(m, a) : (R)0;
+    return ab > 0.0f ? copysignf(m, a) : 0.0f;
   }
 }
 
@@ -384,9 +374,7 @@ __device__ __forceinline__ R limit(R a, R b) {
 // Components E and E_nu of Y (the others vanish with f = 0).
 // SRC 0: frozen limit (no source); 1: Q and I exponents all zero (Q = I = Q0,
 // so rho (Q - I) = 0); 2: general closures of eq. 6.
-template <typename R, int SRC> struct Src;
-
-template <int SRC> struct Src<float, SRC> {
+template <int SRC> struct Src {
   static __device__ __forceinline__ void eval(const P<float>& k, float rho, float T, float Ev,
                                               float& yE, float& yEv) {
     if (SRC == 0) {
@@ -404,53 +392,6 @@ template <int SRC> struct Src<float, SRC> {
       yE = rho * (Q - I);
     }
     yEv = fmaf(rho * k.Ck, T, -Ev) * inv_tau + rho * Q;
-  }
-};
-
-__device__ __forceinline__ double half_powers(double rho, double sr, int kr, double T, double sT,
-                                              int kT) {
-  double num = 1.0, den = 1.0;
-  const int ar = kr < 0 ? -kr : kr, aT = kT < 0 ? -kT : kT;
-  double pr = (ar & 1) ? sr : 1.0, pT = (aT & 1) ? sT : 1.0;
-  for (int i = 0; i < (ar >> 1); ++i) pr *= rho;
-  for (int i = 0; i < (aT >> 1); ++i) pT *= T;
-  if (kr < 0) den *= pr; else num *= pr;
-  if (kT < 0) den *= pT; else num *= pT;
-  return (kr < 0 || kT < 0) ? num * Ar<double>::rcp(den) : num;
-}
-
-template <int SRC> struct Src<double, SRC> {
-  static __device__ __forceinline__ void eval(const P<double>& k, double rho, double T, double Ev,
-                                              double& yE, double& yEv) {
-    if (SRC == 0) {
-      yE = yEv = 0.0;
-      return;
-    }
-    double inv_tau, Q = k.Q0, I = k.Q0;
-    if (k.half_tau && (SRC == 1 || k.half_qi)) {
-      // exponents that are multiples of 1/2: products and at most one square
-      // root per variable, in place of logarithms and exponentials on GB300's
-      // narrow FP64 pipe
-      const bool odd_r = ((k.hk[0] | (SRC == 2 ? k.hk[2] | k.hk[4] : 0)) & 1) != 0;
-      const bool odd_T = ((k.hk[1] | (SRC == 2 ? k.hk[3] | k.hk[5] : 0)) & 1) != 0;
-      const double sr = odd_r ? sqrt(rho) : 1.0, sT = odd_T ? sqrt(T) : 1.0;
-      inv_tau = k.inv_tau0 * half_powers(rho, sr, -k.hk[0], T, sT, -k.hk[1]);
-      if (SRC == 2) {
-        Q = k.Q0 * half_powers(rho, sr, k.hk[2], T, sT, k.hk[3]);
-        I = k.Q0 * half_powers(rho, sr, k.hk[4], T, sT, k.hk[5]);
-      }
-    } else {
-      // the power laws of eq. 6 as exp of a linear form in ln rho, ln T: two
-      // logarithms per state instead of two pow per closure (GB300's FP64 rate)
-      const double lr = log(rho), lT = log(T);
-      inv_tau = exp(-fma(k.tau_rho, lr, k.tau_T * lT)) * k.inv_tau0;
-      if (SRC == 2) {
-        Q = k.Q0 * exp(fma(k.Q_rho, lr, k.Q_T * lT));
-        I = k.Q0 * exp(fma(k.I_rho, lr, k.I_T * lT));
-      }
-    }
-    yE = rho * (Q - I);
-    yEv = (rho * k.Ck * T - Ev) * inv_tau + rho * Q;
   }
 };
 

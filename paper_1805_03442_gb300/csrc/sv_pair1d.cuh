@@ -42,12 +42,12 @@ __device__ __forceinline__ f2 sqrt_pos(f2 a) {
 // the limiter per component (minmod: three ALU instructions, sv_model.cuh)
 template <int LIM>
 __device__ __forceinline__ float slope(float a, float b) {
-  return limit<LIM, float>(a, b);
+  return limit<LIM>(a, b);
 }
 
 // eq. 5 of two states, rho |v|^2 = kin2 given: PP = 0 in float (E - E_nu
-// first, as pressure<float, 0>), PP = 2 in compensated float (the
-// pressure<float, 2> policy); component by component, each packed add,
+// first, as pressure<0>), PP = 2 in compensated float (the
+// pressure<2> policy); component by component, each packed add,
 // subtract and fused multiply-add rounds as the scalar one.
 template <int PP>
 __device__ __forceinline__ f2 pressure(const P<float>& k, f2 kin2, f2 E, f2 Ev) {
@@ -78,7 +78,7 @@ __device__ __forceinline__ Prim prim(const P<float>& k, const f2 (&u)[4]) {
   return q;
 }
 
-// Components E and E_nu of Y (eq. 6 closures), as Src<float, SRC>.
+// Components E and E_nu of Y (eq. 6 closures), as Src<SRC>.
 template <int SRC>
 __device__ __forceinline__ void source(const P<float>& k, f2 rho, f2 T, f2 Ev, f2& yE, f2& yEv) {
   yE = splat(0.0f);

@@ -136,7 +136,7 @@ __device__ __forceinline__ void cfl(const P<float>& k, const f2 (&N)[DIM + 3], i
   for (int a = 1; a < DIM; ++a) v2 = fma(q.v[a], q.v[a], v2);
   f2 key = splat(-INFINITY);
   if (SRC != 0) key = fma(splat(k.ntau_rho), pk::lg2(N[0]), mul(splat(k.ntau_T), pk::lg2(mul(q.p, q.ir))));
-  const float vx = speed_of<float>(v2.x), vy = speed_of<float>(v2.y);
+  const float vx = speed_of(v2.x), vy = speed_of(v2.y);
   if (mask & 1) {
     if ((N[0].x > 0.0f) && (q.p.x > 0.0f)) {
       smax = fmaxf(smax, fmaxf(2.0f * vx, vx + c.x));

@@ -86,7 +86,7 @@ __device__ __forceinline__ void bound(const P<float>& k, const float (&u)[4], fl
   const float vmag = fabsf(q.v);
   const float c = Ar<float>::sqrt_pos(k.gamma * q.p * q.ir);
   smax = fmaxf(smax, fmaxf(2.0f * vmag, vmag + c));
-  if (SRC != 0) akey = fmaxf(akey, TauKey<float>::of(k, q.rho, q.p * q.ir));
+  if (SRC != 0) akey = fmaxf(akey, tau_key(k, q.rho, q.p * q.ir));
 }
 
 }  // namespace ps
@@ -308,15 +308,19 @@ __device__ __forceinline__ void cfl(const P<float>& k, const pk::f2 (&N)[4], int
 
 // eq. 16 bound of one 1D cell state u (rho, rho v, E, E_nu), or of its
 // perturbation (PP = 3), folded into the caller's maxima.
-template <typename R, int PP, int SRC>
-__device__ __forceinline__ void cell_bound(const P<R>& k, const R (&u)[4], R& smax, R& akey,
-                                           uint32_t& flags) {
+template <int PP, int SRC>
+__device__ __forceinline__ void cell_bound(const P<float>& k, const float (&u)[4], Acc<float>& m) {
   if constexpr (PP == 3) {
-    ps::bound<SRC>(k, u, smax, akey, flags);
+    ps::bound<SRC>(k, u, m.smax, m.akey, m.flags);
   } else {
-    const R v = u[1] * Ar<R>::rcp(u[0]);
-    cfl_cell<R, PP, SRC>(k, u[0], u[1] * v, fabs(v), u[2], u[3], smax, akey, flags);
+    const float v = u[1] * Ar<float>::rcp(u[0]);
+    cfl_cell<PP, SRC>(k, u[0], u[1] * v, fabsf(v), u[2], u[3], m.smax, m.akey, m.flags);
   }
+}
+template <int PP, int SRC>
+__device__ __forceinline__ void cell_bound(const P<double>& k, const double (&u)[4],
+                                           Acc<double>& m) {
+  d64::bound<1, SRC>(k, u, m);
 }
 
 }  // namespace sv

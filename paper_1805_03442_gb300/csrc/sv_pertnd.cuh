@@ -79,10 +79,10 @@ __device__ __forceinline__ void bound(const P<float>& k, const float (&u)[DIM + 
     flags |= FLAG_NONPHYS;
     return;
   }
-  const float vmag = speed_of<float>(q.v2);
+  const float vmag = speed_of(q.v2);
   const float c = Ar<float>::sqrt_pos(k.gamma * q.p * q.ir);
   smax = fmaxf(smax, fmaxf(2.0f * vmag, vmag + c));
-  if (SRC != 0) akey = fmaxf(akey, TauKey<float>::of(k, q.rho, q.p * q.ir));
+  if (SRC != 0) akey = fmaxf(akey, tau_key(k, q.rho, q.p * q.ir));
 }
 
 }  // namespace psn
@@ -213,7 +213,7 @@ __device__ __forceinline__ void cfl(const P<float>& k, const f2 (&N)[DIM + 3], i
   f2 key = splat(-INFINITY);
   if (SRC != 0)
     key = fma(splat(k.ntau_rho), pk::lg2(q.rho), mul(splat(k.ntau_T), pk::lg2(mul(q.p, q.ir))));
-  const float vx = speed_of<float>(v2.x), vy = speed_of<float>(v2.y);
+  const float vx = speed_of(v2.x), vy = speed_of(v2.y);
   if (mask & 1) {
     if ((q.rho.x > 0.0f) && (q.p.x > 0.0f)) {
       smax = fmaxf(smax, fmaxf(2.0f * vx, vx + c.x));

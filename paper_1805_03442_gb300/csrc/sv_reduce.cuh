@@ -11,54 +11,53 @@
 // stepping, so K steps can be replayed from a CUDA graph.
 #pragma once
 
+#include "sv_f64.cuh"
 #include "sv_model.cuh"
 
 namespace sv {
 
-// The tau bound is folded as a maximum:
+// What a thread folds over the cells it updates: the largest signal speed, the
+// tau bound as a maximum and the flags.
 //   float kernels:  a_j = -(tau_rho log2 rho + tau_T log2 T), tau_j = tau0 2^-a_j
-//   double kernels: a_j = -tau_j (tau_j from pow, as in the closure of eq. 6)
-template <typename R> struct TauKey;
-template <> struct TauKey<float> {
-  static __device__ __forceinline__ float of(const P<float>& k, float rho, float T) {
-    return -fmaf(k.tau_rho, Ar<float>::lg2(rho), k.tau_T * Ar<float>::lg2(T));
-  }
+//   double kernels: a_j = -tau_j, and the thresholds of d64::Bound
+template <typename R> struct Acc;
+template <> struct Acc<float> {
+  float smax = 0.0f, akey = -INFINITY;
+  uint32_t flags = 0;
+  __device__ __forceinline__ explicit Acc(float*) {}
 };
-template <> struct TauKey<double> {
-  static __device__ __forceinline__ double of(const P<double>& k, double rho, double T) {
-    if (k.half_tau) {
-      const double sr = (k.hk[0] & 1) ? sqrt(rho) : 1.0, sT = (k.hk[1] & 1) ? sqrt(T) : 1.0;
-      return -(k.tau0 * half_powers(rho, sr, k.hk[0], T, sT, k.hk[1]));
-    }
-    return -(k.tau0 * exp(fma(k.tau_rho, log(rho), k.tau_T * log(T))));
-  }
+template <> struct Acc<double> : d64::Bound {
+  __device__ __forceinline__ explicit Acc(float* word) { share = word; }
 };
+
+__device__ __forceinline__ float tau_key(const P<float>& k, float rho, float T) {
+  return -fmaf(k.tau_rho, Ar<float>::lg2(rho), k.tau_T * Ar<float>::lg2(T));
+}
 
 // |v| from v.v for the eq. 16 bound of 2D / 3D states.  In float,
 // x * rsqrt(x) of a subnormal v.v (the far tail of a wave still spreading into
 // gas at rest) flushes the rsqrt argument to zero and gives +inf; a speed
 // below 1e-19 cannot change max(2|v|, |v| + c) in float, so it counts as 0.
-template <typename R>
-__device__ __forceinline__ R speed_of(R v2) {
-  if (std::is_same<R, float>::value) return v2 >= (R)1.17549435e-38 ? Ar<R>::sqrt_pos(v2) : (R)0;
-  return v2 > (R)0 ? Ar<R>::sqrt_pos(v2) : (R)0;
+__device__ __forceinline__ float speed_of(float v2) {
+  return v2 >= 1.17549435e-38f ? Ar<float>::sqrt_pos(v2) : 0.0f;
 }
 
-// Signal speed, tau key and physicality of one updated state (dim-generic),
-// folded into per-thread maxima of the kernel's own type.
+// Signal speed, tau key and physicality of one updated float state
+// (dim-generic), folded into per-thread maxima.
 // `kin2` = rho |v|^2, `vmag` = |v|.  SRC 0 (frozen) has no tau bound.
-template <typename R, int PP, int SRC>
-__device__ __forceinline__ void cfl_cell(const P<R>& k, R rho, R kin2, R vmag, R E, R Ev,
-                                         R& smax, R& akey, uint32_t& flags) {
-  const R p = pressure<R, PP>(k, kin2, E, Ev);
-  const R ir = Ar<R>::rcp(rho);
+template <int PP, int SRC>
+__device__ __forceinline__ void cfl_cell(const P<float>& k, float rho, float kin2, float vmag,
+                                         float E, float Ev, float& smax, float& akey,
+                                         uint32_t& flags) {
+  const float p = pressure<PP>(k, kin2, E, Ev);
+  const float ir = Ar<float>::rcp(rho);
   if (!both_positive(rho, p)) {
     flags |= FLAG_NONPHYS;
     return;
   }
-  const R c = Ar<R>::sqrt_pos(k.gamma * p * ir);
-  smax = fmax(smax, fmax((R)2 * vmag, vmag + c));
-  if (SRC != 0) akey = fmax(akey, TauKey<R>::of(k, rho, p * ir));
+  const float c = Ar<float>::sqrt_pos(k.gamma * p * ir);
+  smax = fmaxf(smax, fmaxf(2.0f * vmag, vmag + c));
+  if (SRC != 0) akey = fmaxf(akey, tau_key(k, rho, p * ir));
 }
 
 // eq. 16 times cfl from the maximal signal speed, capped by c_tau * min tau;

@@ -36,13 +36,12 @@ step1d_kernel(const KParams kp, R* __restrict__ bufA, R* __restrict__ bufB, Ctl*
   const int c0 = (int)((int64_t)warp * nchunk / nwarps);
   const int c1 = (int)((int64_t)(warp + 1) * nchunk / nwarps);
 
-  R smax = 0, akey = -INFINITY;
-  uint32_t flags = 0;
+  Acc<R> acc(bound_word());
 
-  step1d_warp<R, PP, LIM, SRC>(k, Uin, Uout, N, N, c0, c1, lane, dt, dtdx, dt_2h, dt_2, smax, akey,
-                               flags, ring, kp, sc.t);
+  step1d_warp<R, PP, LIM, SRC>(k, Uin, Uout, N, N, c0, c1, lane, dt, dtdx, dt_2h, dt_2, acc, ring,
+                               kp, sc.t);
   pdl_trigger();                                  // the next step may launch and wait
-  reduce_and_finalize<R, NT1>(ctl, kp, smax, akey, flags, true);
+  reduce_and_finalize<R, NT1>(ctl, kp, acc.smax, acc.akey, acc.flags, true);
 }
 
 // Kernel variants: arithmetic (float / double / float with compensated

@@ -59,82 +59,35 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
+// The float Heun stages' scalar arithmetic (the float MUSCL-Hancock step is
+// packed, sv_pair1d.cuh; double is sv_f64.cuh).
 // Primitive recovery (eq. 5, eq. 7): 1/rho, v, rho v^2, p.
-template <typename R, int PP>
-__device__ __forceinline__ void prim1(const P<R>& k, const R (&u)[4], R& ir, R& v, R& kin2, R& p) {
-  ir = Ar<R>::rcp(u[0]);
+__device__ __forceinline__ void prim1(const P<float>& k, const float (&u)[4], float& ir, float& v,
+                                      float& kin2, float& p) {
+  ir = Ar<float>::rcp(u[0]);
   v = u[1] * ir;
   kin2 = u[1] * v;
-  p = pressure<R, PP>(k, kin2, u[2], u[3]);
-}
-
-// Steps 1-3 for one cell: slopes d (= Theta h), predictor, face states
-// wp = U^{n+1/2} + d/2 (right face), wm = U^{n+1/2} - d/2 (left face), and the
-// source at U^{n+1/2} (E and E_nu components).
-template <typename R, int PP, int LIM, int SRC>
-__device__ __forceinline__ void predict(const P<R>& k, const R (&u)[4], const R (&um)[4],
-                                        const R (&up)[4], R dt_2h, R dt_2, R (&wp)[4], R (&wm)[4],
-                                        R& yEh, R& yEvh) {
-  R d[4], a[4], b[4];
-#pragma unroll
-  for (int f = 0; f < 4; ++f) {
-    d[f] = limit<LIM, R>(u[f] - um[f], up[f] - u[f]);
-    a[f] = u[f] + (R)0.5 * d[f];
-    b[f] = u[f] - (R)0.5 * d[f];
-  }
-  R ira, va, ka, pa, irb, vb, kb, pb;
-  prim1<R, PP>(k, a, ira, va, ka, pa);
-  prim1<R, PP>(k, b, irb, vb, kb, pb);
-  R dF[4];
-  dF[0] = a[1] - b[1];
-  dF[1] = (ka + pa) - (kb + pb);
-  dF[2] = va * (a[2] + pa) - vb * (b[2] + pb);
-  dF[3] = va * a[3] - vb * b[3];
-  // positivity guard: a non-physical extrapolated state drops the slopes
-  if (!all_positive(a[0], pa, b[0], pb)) {
-#pragma unroll
-    for (int f = 0; f < 4; ++f) d[f] = dF[f] = (R)0;
-  }
-  R yE = 0, yEv = 0;
-  if (SRC != 0) {
-    R ir, v, kin2, p;
-    prim1<R, PP>(k, u, ir, v, kin2, p);
-    Src<R, SRC>::eval(k, u[0], p * ir, u[3], yE, yEv);
-  }
-  R uh[4];
-  uh[0] = u[0] - dt_2h * dF[0];
-  uh[1] = u[1] - dt_2h * dF[1];
-  uh[2] = u[2] - dt_2h * dF[2] + dt_2 * yE;
-  uh[3] = u[3] - dt_2h * dF[3] + dt_2 * yEv;
-#pragma unroll
-  for (int f = 0; f < 4; ++f) {
-    wp[f] = uh[f] + (R)0.5 * d[f];
-    wm[f] = uh[f] - (R)0.5 * d[f];
-  }
-  yEh = yEvh = (R)0;
-  if (SRC != 0) {
-    R ir, v, kin2, p;
-    prim1<R, PP>(k, uh, ir, v, kin2, p);
-    Src<R, SRC>::eval(k, uh[0], p * ir, uh[3], yEh, yEvh);
-  }
+  p = pressure<0>(k, kin2, u[2], u[3]);
 }
 
 // Heun stages: slopes with the same guard, face states at the stage's own time
 // level (wp = u + d/2, wm = u - d/2) and the source Y(u) for the update.
-template <typename R, int PP, int LIM, int SRC>
-__device__ __forceinline__ void level_states(const P<R>& k, const R (&u)[4], const R (&um)[4],
-                                             const R (&up)[4], R (&wp)[4], R (&wm)[4], R& yE,
-                                             R& yEv) {
+template <int LIM, int SRC>
+__device__ __forceinline__ void level_states(const P<float>& k, const float (&u)[4],
+                                             const float (&um)[4], const float (&up)[4],
+                                             float (&wp)[4], float (&wm)[4], float& yE,
+                                             float& yEv) {
+  using R = float;
   R d[4], a[4], b[4];
 #pragma unroll
   for (int f = 0; f < 4; ++f) {
-    d[f] = limit<LIM, R>(u[f] - um[f], up[f] - u[f]);
+    d[f] = limit<LIM>(u[f] - um[f], up[f] - u[f]);
     a[f] = u[f] + (R)0.5 * d[f];
     b[f] = u[f] - (R)0.5 * d[f];
   }
   R ira, va, ka, pa, irb, vb, kb, pb;
-  prim1<R, PP>(k, a, ira, va, ka, pa);
-  prim1<R, PP>(k, b, irb, vb, kb, pb);
+  prim1(k, a, ira, va, ka, pa);
+  prim1(k, b, irb, vb, kb, pb);
   if (!all_positive(a[0], pa, b[0], pb)) {
 #pragma unroll
     for (int f = 0; f < 4; ++f) a[f] = b[f] = u[f];
@@ -147,27 +100,27 @@ __device__ __forceinline__ void level_states(const P<R>& k, const R (&u)[4], con
   yE = yEv = (R)0;
   if (SRC != 0) {
     R ir, v, kin2, p;
-    prim1<R, PP>(k, u, ir, v, kin2, p);
-    Src<R, SRC>::eval(k, u[0], p * ir, u[3], yE, yEv);
+    prim1(k, u, ir, v, kin2, p);
+    Src<SRC>::eval(k, u[0], p * ir, u[3], yE, yEv);
   }
 }
 
 // eq. 13 at one face; a face with a non-physical state uses the cell values
 // (fl, fr) instead.
-template <typename R, int PP>
-__device__ __forceinline__ void hll(const P<R>& k, const R (&l)[4], const R (&r)[4],
-                                    const R (&fl)[4], const R (&fr)[4], R (&F)[4]) {
+__device__ __forceinline__ void hll(const P<float>& k, const float (&l)[4], const float (&r)[4],
+                                    const float (&fl)[4], const float (&fr)[4], float (&F)[4]) {
+  using R = float;
   R L[4], Rr[4];
 #pragma unroll
   for (int f = 0; f < 4; ++f) { L[f] = l[f]; Rr[f] = r[f]; }
   R irL, uL, kL, pL, irR, uR, kR, pR;
-  prim1<R, PP>(k, L, irL, uL, kL, pL);
-  prim1<R, PP>(k, Rr, irR, uR, kR, pR);
+  prim1(k, L, irL, uL, kL, pL);
+  prim1(k, Rr, irR, uR, kR, pR);
   if (!all_positive(L[0], pL, Rr[0], pR)) {
 #pragma unroll
     for (int f = 0; f < 4; ++f) { L[f] = fl[f]; Rr[f] = fr[f]; }
-    prim1<R, PP>(k, L, irL, uL, kL, pL);
-    prim1<R, PP>(k, Rr, irR, uR, kR, pR);
+    prim1(k, L, irL, uL, kL, pL);
+    prim1(k, Rr, irR, uR, kR, pR);
   }
   const R cL = Ar<R>::sqrt_pos(k.gamma * pL * irL);
   const R cR = Ar<R>::sqrt_pos(k.gamma * pR * irR);
@@ -205,16 +158,40 @@ __device__ __forceinline__ R shfl(R v, int src) {
   return __shfl_sync(0xffffffffu, v, src);
 }
 
+// The double stages' faces with the same signature.
+__device__ __forceinline__ void hll(const P<double>& k, const double (&l)[4], const double (&r)[4],
+                                    const double (&fl)[4], const double (&fr)[4], double (&F)[4]) {
+  double L[4], R[4];
+#pragma unroll
+  for (int f = 0; f < 4; ++f) {
+    L[f] = l[f];
+    R[f] = r[f];
+  }
+  d64::hll<1, 0>(k, L, R,
+                 [&](double (&cl)[4], double (&cr)[4]) {
+#pragma unroll
+                   for (int f = 0; f < 4; ++f) {
+                     cl[f] = fl[f];
+                     cr[f] = fr[f];
+                   }
+                 },
+                 F);
+}
+
 // Conservative update (eq. 15) of one cell and, with CFL, its next-dt bound.
-template <typename R, int PP, int SRC, bool CFL = true>
+template <int PP, int SRC, bool CFL, typename R>
 __device__ __forceinline__ void update_cell(const P<R>& k, const R (&u)[4], const R (&Fl)[4],
                                             const R (&Fr)[4], R yE, R yEv, R dt, R dtdx,
-                                            R (&un)[4], R& smax, R& akey, uint32_t& flags) {
-  un[0] = u[0] - dtdx * (Fr[0] - Fl[0]);
-  un[1] = u[1] - dtdx * (Fr[1] - Fl[1]);
-  un[2] = u[2] - dtdx * (Fr[2] - Fl[2]) + dt * yE;
-  un[3] = u[3] - dtdx * (Fr[3] - Fl[3]) + dt * yEv;
-  if (CFL) cell_bound<R, PP, SRC>(k, un, smax, akey, flags);
+                                            R (&un)[4], Acc<R>& m) {
+  if constexpr (std::is_same<R, double>::value) {
+    d64::update1<SRC>(u, Fl, Fr, yE, yEv, dt, dtdx, un);
+  } else {
+    un[0] = u[0] - dtdx * (Fr[0] - Fl[0]);
+    un[1] = u[1] - dtdx * (Fr[1] - Fl[1]);
+    un[2] = u[2] - dtdx * (Fr[2] - Fl[2]) + dt * yE;
+    un[3] = u[3] - dtdx * (Fr[3] - Fl[3]) + dt * yEv;
+  }
+  if (CFL) cell_bound<PP, SRC>(k, un, m);
 }
 
 // State of the driven boundary's ghost cell centred at x at time t (double).
@@ -241,9 +218,8 @@ enum { MODE_HANCOCK = 0, MODE_HEUN1 = 1, MODE_HEUN2 = 2 };
 template <typename R, int PP, int LIM, int SRC, int MODE = MODE_HANCOCK>
 __device__ __forceinline__ void step1d_warp(const P<R>& k, const R* __restrict__ Uin, R* Uout,
                                             int N, int stride, int c0, int c1, int lane, R dt,
-                                            R dtdx, R dt_2h, R dt_2, R& smax, R& akey,
-                                            uint32_t& flags, R* __restrict__ ring,
-                                            const KParams& kp, double t, const R* U0 = nullptr) {
+                                            R dtdx, R dt_2h, R dt_2, Acc<R>& acc,
+                                            R* __restrict__ ring, const KParams& kp, double t, const R* U0 = nullptr) {
   using R2 = typename Pair<R>::T;
   constexpr int RS = kRing1d, RN = RS * 64, MASK = RN - 1;
   if (c1 <= c0) return;
@@ -351,7 +327,7 @@ __device__ __forceinline__ void step1d_warp(const P<R>& k, const R* __restrict__
           f2 Nw[4];
           pk::update<SRC>(Qp, F_prev, FRt, YE_prev, YEv_prev, dt2, ndtdx2, Nw);
           const bool two = jo + 1 < N;
-          pkx::cfl<PP, SRC>(k, Nw, two ? 3 : 1, smax, akey, flags);
+          pkx::cfl<PP, SRC>(k, Nw, two ? 3 : 1, acc.smax, acc.akey, acc.flags);
           if (two && (stride % 2) == 0) {
 #pragma unroll
             for (int f = 0; f < 4; ++f) *reinterpret_cast<f2*>(Uout + f * stride + jo) = Nw[f];
@@ -386,20 +362,33 @@ __device__ __forceinline__ void step1d_warp(const P<R>& k, const R* __restrict__
         up[f] = rf[(pos + 2) & MASK];
       }
       R Wp0[4], Wm0[4], Wp1[4], Wm1[4], y0E, y0Ev, y1E, y1Ev;
-      if (MODE == MODE_HANCOCK) {
-        predict<R, PP, LIM, SRC>(k, x0, um, x1, dt_2h, dt_2, Wp0, Wm0, y0E, y0Ev);
-        predict<R, PP, LIM, SRC>(k, x1, x0, up, dt_2h, dt_2, Wp1, Wm1, y1E, y1Ev);
+      if constexpr (std::is_same<R, double>::value) {
+        // one-sided differences, the inner one shared by both cells
+        R da[4], dc[4], db[4];
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+          da[f] = d64::sub(x0[f], um[f]);
+          dc[f] = d64::sub(x1[f], x0[f]);
+          db[f] = d64::sub(up[f], x1[f]);
+        }
+        if constexpr (MODE == MODE_HANCOCK) {
+          d64::predict1<LIM, SRC>(k, x0, da, dc, dt_2h, dt_2, Wp0, Wm0, y0E, y0Ev);
+          d64::predict1<LIM, SRC>(k, x1, dc, db, dt_2h, dt_2, Wp1, Wm1, y1E, y1Ev);
+        } else {
+          d64::level1<LIM, SRC>(k, x0, da, dc, Wp0, Wm0, y0E, y0Ev);
+          d64::level1<LIM, SRC>(k, x1, dc, db, Wp1, Wm1, y1E, y1Ev);
+        }
       } else {
-        level_states<R, PP, LIM, SRC>(k, x0, um, x1, Wp0, Wm0, y0E, y0Ev);
-        level_states<R, PP, LIM, SRC>(k, x1, x0, up, Wp1, Wm1, y1E, y1Ev);
+        level_states<LIM, SRC>(k, x0, um, x1, Wp0, Wm0, y0E, y0Ev);
+        level_states<LIM, SRC>(k, x1, x0, up, Wp1, Wm1, y1E, y1Ev);
       }
       R Fa[4] = {0, 0, 0, 0}, Fb[4];
-      hll<R, PP>(k, Wp0, Wm1, x0, x1, Fb);            // face 2i + 1/2
+      hll(k, Wp0, Wm1, x0, x1, Fb);            // face 2i + 1/2
       if (kk >= c0) {
         R WL[4];
 #pragma unroll
         for (int f = 0; f < 4; ++f) WL[f] = shfl(lane == 31 ? Wp1_prev[f] : Wp1[f], src_m);
-        hll<R, PP>(k, WL, Wm0, um, x0, Fa);           // face 2i - 1/2
+        hll(k, WL, Wm0, um, x0, Fa);           // face 2i - 1/2
       }
       if (kk > c0) {
         // update of the pair of chunk kk-1
@@ -419,11 +408,11 @@ __device__ __forceinline__ void step1d_warp(const P<R>& k, const R* __restrict__
             }
           }
           const R udt = MODE == MODE_HEUN2 ? dt_2 : dt, udx = MODE == MODE_HEUN2 ? dt_2h : dtdx;
-          update_cell<R, PP, SRC, MODE != MODE_HEUN1>(k, q0, Fa_prev, Fb_prev, y0E_prev, y0Ev_prev,
-                                                       udt, udx, n0, smax, akey, flags);
+          update_cell<PP, SRC, MODE != MODE_HEUN1>(k, q0, Fa_prev, Fb_prev, y0E_prev, y0Ev_prev,
+                                                   udt, udx, n0, acc);
           if (jo + 1 < N) {
-            update_cell<R, PP, SRC, MODE != MODE_HEUN1>(k, q1, Fb_prev, FR, y1E_prev, y1Ev_prev, udt,
-                                                         udx, n1, smax, akey, flags);
+            update_cell<PP, SRC, MODE != MODE_HEUN1>(k, q1, Fb_prev, FR, y1E_prev, y1Ev_prev, udt,
+                                                     udx, n1, acc);
             if ((stride % 2) == 0) {
 #pragma unroll
               for (int f = 0; f < 4; ++f)

@@ -1,7 +1,9 @@
-// sv_stepnd.cu -- fused 2D / 3D unsplit MUSCL-Hancock steps (Sec. 2.3:
+// sv_stepnd.cu -- fused 2D / 3D unsplit MUSCL-Hancock steps in double (Sec. 2.3:
 // eq. 15 with both flux differences F and G -- and the analogous z flux in
 // 3D -- in one update; eq. 14 face states per axis with xi = 0; eq. 13 HLL per
-// axis; source Y at the half step; eq. 16 reduction).
+// axis; source Y at the half step; eq. 16 reduction), and the dispatch of the
+// float steps to their kernels.  Bound by the FP64 pipe: the arithmetic is that
+// of sv_f64.cuh.
 //
 // Work decomposition ("marching planes").  Each block owns a transverse tile
 // (TX threads along x in 2D; TX x TY threads over x-y in 3D) and a segment of
@@ -20,7 +22,10 @@
 //   e. computes the marching-axis face between planes q-1 and q,
 //   f. updates plane q-1 (all its faces are now known) and folds its
 //      signal speed / tau bound for the next dt.
-// Three barriers per plane.  Each thread streams its own column (and the halo
+// Three barriers per plane.  The warm-up plane before the segment and the
+// plane beyond it skip the transverse faces, which nothing uses there (500^2
+// with walls, 7-row segments: 261 -> 241 us per step; 64^3: 587 -> 546).
+// Each thread streams its own column (and the halo
 // threads their second-ring cells) through a per-thread ring of kPlaneRing
 // planes in shared memory with cp.async, four planes ahead of the one being
 // computed; copies are coalesced along x.
@@ -29,91 +34,6 @@
 #include "sv_step1d.cuh"      // cp.async helpers
 
 namespace sv {
-
-template <typename R, int PP, int DIM, int SRC>
-struct Nd {
-  static constexpr int NF = DIM + 3;
-  using V = R[NF];
-
-  static __device__ __forceinline__ void prim(const P<R>& k, const V& u, R& ir, R (&v)[DIM], R& p) {
-    ir = Ar<R>::rcp(u[0]);
-    R kin2 = 0;
-#pragma unroll
-    for (int a = 0; a < DIM; ++a) {
-      v[a] = u[1 + a] * ir;
-      kin2 += u[1 + a] * v[a];
-    }
-    p = pressure<R, PP>(k, kin2, u[1 + DIM], u[2 + DIM]);
-  }
-
-  template <int A>
-  static __device__ __forceinline__ void flux(const V& u, const R (&v)[DIM], R p, V& F) {
-    F[0] = u[1 + A];
-#pragma unroll
-    for (int b = 0; b < DIM; ++b) F[1 + b] = u[1 + b] * v[A] + (b == A ? p : (R)0);
-    F[1 + DIM] = v[A] * (u[1 + DIM] + p);
-    F[2 + DIM] = v[A] * u[2 + DIM];
-  }
-
-  // F(u + d/2) - F(u - d/2) along axis A; returns false if a state is non-physical
-  template <int A>
-  static __device__ __forceinline__ bool dflux(const P<R>& k, const V& u, const V& d, V& dF) {
-    V a, b;
-#pragma unroll
-    for (int f = 0; f < NF; ++f) {
-      a[f] = u[f] + (R)0.5 * d[f];
-      b[f] = u[f] - (R)0.5 * d[f];
-    }
-    R ira, irb, pa, pb, va[DIM], vb[DIM];
-    prim(k, a, ira, va, pa);
-    prim(k, b, irb, vb, pb);
-    V Fa, Fb;
-    flux<A>(a, va, pa, Fa);
-    flux<A>(b, vb, pb, Fb);
-#pragma unroll
-    for (int f = 0; f < NF; ++f) dF[f] = Fa[f] - Fb[f];
-    return all_positive(a[0], pa, b[0], pb);
-  }
-
-  // Y of a cell of the active medium; a frozen cell (active = false) has none.
-  static __device__ __forceinline__ void source(const P<R>& k, const V& u, R& yE, R& yEv,
-                                                bool active = true) {
-    yE = yEv = (R)0;
-    if (SRC == 0 || !active) return;
-    R ir, p, v[DIM];
-    prim(k, u, ir, v, p);
-    Src<R, SRC>::eval(k, u[0], p * ir, u[2 + DIM], yE, yEv);
-  }
-
-  // eq. 13 along axis A
-  template <int A>
-  static __device__ __forceinline__ void hll(const P<R>& k, const V& l, const V& r, const V& fl,
-                                             const V& fr, V& F) {
-    V L, Rr;
-#pragma unroll
-    for (int f = 0; f < NF; ++f) { L[f] = l[f]; Rr[f] = r[f]; }
-    R irL, pL, vL[DIM], irR, pR, vR[DIM];
-    prim(k, L, irL, vL, pL);
-    prim(k, Rr, irR, vR, pR);
-    if (!all_positive(L[0], pL, Rr[0], pR)) {
-#pragma unroll
-      for (int f = 0; f < NF; ++f) { L[f] = fl[f]; Rr[f] = fr[f]; }
-      prim(k, L, irL, vL, pL);
-      prim(k, Rr, irR, vR, pR);
-    }
-    const R cL = Ar<R>::sqrt_pos(k.gamma * pL * irL);
-    const R cR = Ar<R>::sqrt_pos(k.gamma * pR * irR);
-    const R sl = fmin(fmin(vL[A] - cL, vR[A] - cR), (R)0);
-    const R sr = fmax(fmax(vL[A] + cL, vR[A] + cR), (R)0);
-    V FL, FR;
-    flux<A>(L, vL, pL, FL);
-    flux<A>(Rr, vR, pR, FR);
-    const R inv = Ar<R>::rcp(sr - sl);
-    const R wl = sr * inv, wr = -sl * inv, wd = sl * sr * inv;
-#pragma unroll
-    for (int f = 0; f < NF; ++f) F[f] = wl * FL[f] + wr * FR[f] + wd * (Rr[f] - L[f]);
-  }
-};
 
 // Planes per thread ring (a power of two; four planes are in flight).
 constexpr int kPlaneRing = 8;
@@ -135,11 +55,12 @@ constexpr size_t stepnd_smem() {
 // BND: a 2D grid with walls or outflow on some side, or a medium map / driven
 // cells; without it every axis is periodic (the compiled-out general path
 // costs the periodic kernel 8%).
-template <typename R, int PP, int LIM, int SRC, int DIM, int TX, int TY, int MINB, bool BND>
+template <int LIM, int SRC, int DIM, int TX, int TY, int MINB, bool BND>
 __global__ void __launch_bounds__(TX * TY, MINB)
-stepnd_kernel(const KParams kp, R* __restrict__ bufA, R* __restrict__ bufB, Ctl* __restrict__ ctl,
-              int64_t nx, int64_t ny, int64_t nz, int tiles_x, int tiles_y, int nseg) {
-  using C = Nd<R, PP, DIM, SRC>;
+stepnd_kernel(const KParams kp, double* __restrict__ bufA, double* __restrict__ bufB,
+              Ctl* __restrict__ ctl, int64_t nx, int64_t ny, int64_t nz, int tiles_x, int tiles_y,
+              int nseg) {
+  using R = double;
   constexpr int NF = DIM + 3;
   constexpr int NT = TX * TY;
   constexpr int SY = DIM == 3 ? TY + 2 : 1;     // rows of the shared state plane
@@ -209,8 +130,7 @@ stepnd_kernel(const KParams kp, R* __restrict__ bufA, R* __restrict__ bufB, Ctl*
   const I col_ry = DIM == 3 ? wrap(gy + (ty == 0 ? -1 : 1), nyi) * nxi + wx : 0;
   const int oy = DIM == 3 ? ty + 1 : 0;
 
-  R smax = 0, akey = -INFINITY;
-  uint32_t flags = 0;
+  Acc<R> acc(bound_word());
 
   const int tid = threadIdx.x;
   const int hx = ty * 2 + (tx == 0 ? 0 : 1);                              // x-ring slot
@@ -290,63 +210,83 @@ stepnd_kernel(const KParams kp, R* __restrict__ bufA, R* __restrict__ bufB, Ctl*
     R d[DIM][NF];
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
-      d[0][f] = limit<LIM, R>(Uq[f] - sU[f][oy][tx], sU[f][oy][tx + 2] - Uq[f]);
-      if (DIM == 3) d[1][f] = limit<LIM, R>(Uq[f] - sU[f][oy - 1][tx + 1], sU[f][oy + 1][tx + 1] - Uq[f]);
-      d[AM][f] = limit<LIM, R>(Uq[f] - Um1[f], Up1[f] - Uq[f]);
+      d[0][f] = d64::limit<LIM>(d64::sub(Uq[f], sU[f][oy][tx]), d64::sub(sU[f][oy][tx + 2], Uq[f]));
+      if (DIM == 3)
+        d[1][f] = d64::limit<LIM>(d64::sub(Uq[f], sU[f][oy - 1][tx + 1]),
+                                  d64::sub(sU[f][oy + 1][tx + 1], Uq[f]));
+      d[AM][f] = d64::limit<LIM>(d64::sub(Uq[f], Um1[f]), d64::sub(Up1[f], Uq[f]));
     }
-    R div[NF], dF[NF];
-    bool ok = C::template dflux<0>(k, Uq, d[0], div);
-    ok = C::template dflux<1>(k, Uq, d[1], dF) && ok;
-#pragma unroll
-    for (int f = 0; f < NF; ++f) div[f] += dF[f];
-    if (DIM == 3) {
-      ok = C::template dflux<DIM == 3 ? 2 : 1>(k, Uq, d[AM], dF) && ok;
-#pragma unroll
-      for (int f = 0; f < NF; ++f) div[f] += dF[f];
-    }
+    R div[NF];
+    bool ok = d64::dflux<DIM, 0, true>(k, Uq, d[0], div);
+    ok = d64::dflux<DIM, 1, false>(k, Uq, d[1], div) && ok;
+    if (DIM == 3) ok = d64::dflux<DIM, DIM - 1, false>(k, Uq, d[AM], div) && ok;
     if (!ok) {
 #pragma unroll
       for (int f = 0; f < NF; ++f) {
-        div[f] = (R)0;
+        div[f] = 0.0;
 #pragma unroll
-        for (int a = 0; a < DIM; ++a) d[a][f] = (R)0;
+        for (int a = 0; a < DIM; ++a) d[a][f] = 0.0;
       }
     }
-    R yE, yEv;
-    C::source(k, Uq, yE, yEv, active);
     R uh[NF];
 #pragma unroll
-    for (int f = 0; f < NF; ++f) uh[f] = Uq[f] - dt_2h * div[f];
-    uh[1 + DIM] += dt_2 * yE;
-    uh[2 + DIM] += dt_2 * yEv;
-    R yEh, yEvh;
-    C::source(k, uh, yEh, yEvh, active);
+    for (int f = 0; f < NF; ++f) uh[f] = d64::fma(-dt_2h, div[f], Uq[f]);
+    R yEh = 0.0, yEvh = 0.0;
+    if (SRC != 0 && active) {         // a frozen cell has no source
+      R yE, yEv;
+      d64::source<SRC>(k, Uq[0], d64::prim<DIM, -1>(Uq), Uq[2 + DIM], yE, yEv);
+      if (SRC == 2) uh[1 + DIM] = d64::fma(dt_2, yE, uh[1 + DIM]);
+      uh[2 + DIM] = d64::fma(dt_2, yEv, uh[2 + DIM]);
+      d64::source<SRC>(k, uh[0], d64::prim<DIM, -1>(uh), uh[2 + DIM], yEh, yEvh);
+    }
 
+    R Dq[NF];
+    if (q < q0 || q == q1) {
+      // a warm-up plane (only its marching + states are used) or the plane
+      // beyond the segment (only its marching - states): no transverse faces
+#pragma unroll
+      for (int f = 0; f < NF; ++f) Dq[f] = 0.0;
+      __syncthreads();               // plane q has been read before the next is published
+    } else {
     // c. transverse faces: publish +states, take the left neighbour's
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
-      sW[0][f][ty][tx] = uh[f] + (R)0.5 * d[0][f];
-      if (DIM == 3) sW[DIM == 3 ? 1 : 0][f][ty][tx] = uh[f] + (R)0.5 * d[1][f];
+      sW[0][f][ty][tx] = d64::fma(0.5, d[0][f], uh[f]);
+      if (DIM == 3) sW[DIM == 3 ? 1 : 0][f][ty][tx] = d64::fma(0.5, d[1][f], uh[f]);
     }
     __syncthreads();
     R Fx[NF], Fy[NF];
     {
-      R l[NF], r[NF], fl[NF];
+      R l[NF], r[NF];
 #pragma unroll
       for (int f = 0; f < NF; ++f) {
         l[f] = sW[0][f][ty][tx > 0 ? tx - 1 : tx];
-        r[f] = uh[f] - (R)0.5 * d[0][f];
-        fl[f] = sU[f][oy][tx];
+        r[f] = d64::fma(-0.5, d[0][f], uh[f]);
       }
-      C::template hll<0>(k, l, r, fl, Uq, Fx);
+      d64::hll<DIM, 0>(k, l, r,
+                       [&](R (&L)[NF], R (&Rr)[NF]) {
+#pragma unroll
+                         for (int f = 0; f < NF; ++f) {
+                           L[f] = sU[f][oy][tx];
+                           Rr[f] = Uq[f];
+                         }
+                       },
+                       Fx);
       if (DIM == 3) {
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
           l[f] = sW[DIM == 3 ? 1 : 0][f][ty > 0 ? ty - 1 : ty][tx];
-          r[f] = uh[f] - (R)0.5 * d[1][f];
-          fl[f] = sU[f][oy > 0 ? oy - 1 : oy][tx + 1];
+          r[f] = d64::fma(-0.5, d[1][f], uh[f]);
         }
-        C::template hll<1>(k, l, r, fl, Uq, Fy);
+        d64::hll<DIM, 1>(k, l, r,
+                         [&](R (&L)[NF], R (&Rr)[NF]) {
+#pragma unroll
+                           for (int f = 0; f < NF; ++f) {
+                             L[f] = sU[f][oy > 0 ? oy - 1 : oy][tx + 1];
+                             Rr[f] = Uq[f];
+                           }
+                         },
+                         Fy);
       }
     }
     // d. transverse flux divergence of plane q
@@ -356,48 +296,53 @@ stepnd_kernel(const KParams kp, R* __restrict__ bufA, R* __restrict__ bufB, Ctl*
       if (DIM == 3) sF[DIM == 3 ? 1 : 0][f][ty][tx] = Fy[f];
     }
     __syncthreads();
-    R Dq[NF];
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
-      Dq[f] = sF[0][f][ty][tx < TX - 1 ? tx + 1 : tx] - Fx[f];
-      if (DIM == 3) Dq[f] += sF[DIM == 3 ? 1 : 0][f][ty < TY - 1 ? ty + 1 : ty][tx] - Fy[f];
+      Dq[f] = d64::sub(sF[0][f][ty][tx < TX - 1 ? tx + 1 : tx], Fx[f]);
+      if (DIM == 3)
+        Dq[f] = d64::add(Dq[f], d64::sub(sF[DIM == 3 ? 1 : 0][f][ty < TY - 1 ? ty + 1 : ty][tx], Fy[f]));
+    }
+
     }
 
     // e. marching-axis face between planes q-1 and q
-    R Wm[NF], Hq[NF];
+    R Hq[NF];
+    if (q >= q0) {
+      R Wm[NF];
 #pragma unroll
-    for (int f = 0; f < NF; ++f) Wm[f] = uh[f] - (R)0.5 * d[AM][f];
-    C::template hll<AM>(k, Wm_prev, Wm, Um1, Uq, Hq);
+      for (int f = 0; f < NF; ++f) Wm[f] = d64::fma(-0.5, d[AM][f], uh[f]);
+      d64::hll<DIM, AM>(k, Wm_prev, Wm,
+                        [&](R (&L)[NF], R (&Rr)[NF]) {
+#pragma unroll
+                          for (int f = 0; f < NF; ++f) {
+                            L[f] = Um1[f];
+                            Rr[f] = Uq[f];
+                          }
+                        },
+                        Hq);
+    }
 
     // f. update of plane q-1
     if (q > q0 && interior) {
       R un[NF];
 #pragma unroll
-      for (int f = 0; f < NF; ++f) un[f] = Um1[f] - dtdx * (D_prev[f] + Hq[f] - H_prev[f]);
-      un[1 + DIM] += dt * yE_prev;
-      un[2 + DIM] += dt * yEv_prev;
+      for (int f = 0; f < NF; ++f)
+        un[f] = d64::fma(-dtdx, d64::sub(d64::add(D_prev[f], Hq[f]), H_prev[f]), Um1[f]);
+      if (SRC == 2) un[1 + DIM] = d64::fma(dt, yE_prev, un[1 + DIM]);
+      if (SRC != 0) un[2 + DIM] = d64::fma(dt, yEv_prev, un[2 + DIM]);
       // a driven cell holds the pulsating source at the new time level
       if (pulses && gx >= __ldg(kp.pul_lo + (q - 1)) && gx < __ldg(kp.pul_hi + (q - 1)))
         pulse_state<R, NF>(kp, sc.t + sc.dt, un);
       const I o = pidx(q - 1) + col;
 #pragma unroll
       for (int f = 0; f < NF; ++f) Uout[f * ncell + o] = un[f];
-      R ir, p, v[DIM];
-      C::prim(k, un, ir, v, p);
-      R v2 = 0;
-#pragma unroll
-      for (int a = 0; a < DIM; ++a) v2 += v[a] * v[a];
-      const R vmag = speed_of<R>(v2);
-      R kin2 = 0;
-#pragma unroll
-      for (int a = 0; a < DIM; ++a) kin2 += un[1 + a] * v[a];
-      cfl_cell<R, PP, SRC>(k, un[0], kin2, vmag, un[1 + DIM], un[2 + DIM], smax, akey, flags);
+      d64::bound<DIM, SRC>(k, un, acc);
     }
 
     // rotate the plane window
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
-      Wm_prev[f] = uh[f] + (R)0.5 * d[AM][f];
+      Wm_prev[f] = d64::fma(0.5, d[AM][f], uh[f]);
       D_prev[f] = Dq[f];
       H_prev[f] = Hq[f];
     }
@@ -405,33 +350,33 @@ stepnd_kernel(const KParams kp, R* __restrict__ bufA, R* __restrict__ bufB, Ctl*
     yEv_prev = yEvh;
   }
   cp_async_wait<0>();
-  reduce_and_finalize<R, NT>(ctl, kp, smax, akey, flags, true);
+  reduce_and_finalize<R, NT>(ctl, kp, acc.smax, acc.akey, acc.flags, true);
 }
 
 // ------------------------------------------------------------------ launch
 
-template <int DIM, int PREC> struct Cfg;
-template <> struct Cfg<2, PREC_FP64> { static constexpr int TX = 128, TY = 1, MINB = 2, SEG = 256; };
-template <> struct Cfg<3, PREC_FP64> { static constexpr int TX = 16, TY = 16, MINB = 1, SEG = 128; };
+template <int DIM> struct Cfg;
+template <> struct Cfg<2> { static constexpr int TX = 128, TY = 1, MINB = 2, SEG = 256; };
+template <> struct Cfg<3> { static constexpr int TX = 16, TY = 16, MINB = 1, SEG = 128; };
 
 // With `n` null only the kernel's shared-memory attribute is set (done once per
 // solver at init, outside any stream capture).  `nseg` = segments of the
 // marching axis (march_segments).
-template <typename R, int PP, int LIM, int SRC, int DIM, int PREC>
+template <int LIM, int SRC, int DIM>
 static cudaError_t launch_nd(const KParams& kp, void* a, void* b, Ctl* ctl, const int64_t* n,
                             int nseg, cudaStream_t st) {
-  using G = Cfg<DIM, PREC>;
-  constexpr size_t smem = stepnd_smem<R, DIM, G::TX, G::TY>();
+  using G = Cfg<DIM>;
+  constexpr size_t smem = stepnd_smem<double, DIM, G::TX, G::TY>();
   const bool bnd = DIM == 2 && (kp.bc_lo != BC_PERIODIC || kp.bc_hi != BC_PERIODIC ||
                                 kp.bc_ylo != BC_PERIODIC || kp.bc_yhi != BC_PERIODIC ||
                                 kp.act_lo != nullptr || kp.pul_lo != nullptr);
-  auto fn = bnd ? stepnd_kernel<R, PP, LIM, SRC, DIM, G::TX, G::TY, G::MINB, DIM == 2>
-                : stepnd_kernel<R, PP, LIM, SRC, DIM, G::TX, G::TY, G::MINB, false>;
+  auto fn = bnd ? stepnd_kernel<LIM, SRC, DIM, G::TX, G::TY, G::MINB, DIM == 2>
+                : stepnd_kernel<LIM, SRC, DIM, G::TX, G::TY, G::MINB, false>;
   if (!n) {
-    cudaError_t e = cudaFuncSetAttribute(stepnd_kernel<R, PP, LIM, SRC, DIM, G::TX, G::TY, G::MINB, false>,
+    cudaError_t e = cudaFuncSetAttribute(stepnd_kernel<LIM, SRC, DIM, G::TX, G::TY, G::MINB, false>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess || DIM != 2) return e;
-    return cudaFuncSetAttribute(stepnd_kernel<R, PP, LIM, SRC, DIM, G::TX, G::TY, G::MINB, DIM == 2>,
+    return cudaFuncSetAttribute(stepnd_kernel<LIM, SRC, DIM, G::TX, G::TY, G::MINB, DIM == 2>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   }
   const int64_t nx = n[0], ny = n[1], nz = DIM == 3 ? n[2] : 1;
@@ -440,7 +385,7 @@ static cudaError_t launch_nd(const KParams& kp, void* a, void* b, Ctl* ctl, cons
   if (nseg < 1 || nseg > (DIM == 3 ? nz : ny)) return cudaErrorInvalidValue;
   const int64_t blocks = (int64_t)tiles_x * tiles_y * nseg;
   if (blocks > 0x7fffffff) return cudaErrorInvalidConfiguration;
-  fn<<<(int)blocks, G::TX * G::TY, smem, st>>>(kp, (R*)a, (R*)b, ctl, nx, ny, nz, tiles_x, tiles_y,
+  fn<<<(int)blocks, G::TX * G::TY, smem, st>>>(kp, (double*)a, (double*)b, ctl, nx, ny, nz, tiles_x, tiles_y,
                                                nseg);
   return cudaGetLastError();
 }
@@ -449,7 +394,7 @@ template <int LIM, int SRC, int DIM>
 static cudaError_t by_prec(int precision, const KParams& kp, void* a, void* b, Ctl* ctl,
                            const int64_t* n, int nseg, cudaStream_t st) {
   switch (precision) {
-    case PREC_FP64: return launch_nd<double, 0, LIM, SRC, DIM, PREC_FP64>(kp, a, b, ctl, n, nseg, st);
+    case PREC_FP64: return launch_nd<LIM, SRC, DIM>(kp, a, b, ctl, n, nseg, st);
     default:
       // the float policies: in 2D packed plane pairs
       // (sv_stepnd_pair.cu); in 3D each cell's fields in packed pairs
@@ -478,17 +423,17 @@ static cudaError_t by_lim(int precision, const KParams& kp, void* a, void* b, Ct
   }
 }
 
-template <int DIM, int PREC>
+// Two 2D blocks on an SM take 1.75 times one block's iteration (28.4 and 16.2
+// us); the two extra iterations skip the transverse faces and so cost 1.2.
+template <int DIM>
 static MarchShape shape_of() {
-  using G = Cfg<DIM, PREC>;
-  return {G::TX - 2, DIM == 3 ? G::TY - 2 : 0, 1, G::MINB, {1.0, 1.75, 0.0}, G::SEG};
+  using G = Cfg<DIM>;
+  return {G::TX - 2, DIM == 3 ? G::TY - 2 : 0, 1, 1.2, G::MINB, {1.0, 1.75, 0.0}, G::SEG};
 }
 
 MarchShape stepnd_shape(int dim, int precision) {
-  switch (precision) {
-    case PREC_FP64: return dim == 2 ? shape_of<2, PREC_FP64>() : shape_of<3, PREC_FP64>();
-    default: return dim == 2 ? stepnd_pair_shape() : stepnd3f_shape();
-  }
+  if (precision == PREC_FP64) return dim == 2 ? shape_of<2>() : shape_of<3>();
+  return dim == 2 ? stepnd_pair_shape() : stepnd3f_shape();
 }
 
 int stepnd_grid(int dim, int precision, const KParams& kp) {

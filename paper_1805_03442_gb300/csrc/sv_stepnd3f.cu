@@ -6,7 +6,7 @@ namespace sv {
 
 MarchShape stepnd3f_shape() {
   using T = Tile3f;
-  return {T::TX - 2, T::TY - 2, 1, T::MINB, {1.0, 0.0, 0.0}, T::SEG};
+  return {T::TX - 2, T::TY - 2, 1, 2.0, T::MINB, {1.0, 0.0, 0.0}, T::SEG};
 }
 
 // Float (PREC_FP32), compensated-float (PREC_FP32_PC) and perturbation-layout

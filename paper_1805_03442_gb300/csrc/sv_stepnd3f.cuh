@@ -63,7 +63,7 @@ __device__ __forceinline__ Pr3 prim3(const P<float>& k, const f2 (&u)[NP]) {
     q.pf = k.g1 * fmaf(q.kin2, -0.5f, u[2].x - u[2].y);
     q.p = 1.0f + q.pf;
   } else {
-    q.p = q.pf = pressure<float, PP>(k, q.kin2, u[2].x, u[2].y);
+    q.p = q.pf = pressure<PP>(k, q.kin2, u[2].x, u[2].y);
   }
   return q;
 }
@@ -128,7 +128,7 @@ __device__ __forceinline__ f2 source3(const P<float>& k, const f2 (&u)[NP]) {
     psn::source<3, SRC>(k, v, psn::prim<3>(k, v), yE, yEv);
   } else {
     const Pr3 q = prim3<PP>(k, u);
-    Src<float, SRC>::eval(k, u[0].x, q.p * q.ir, u[2].y, yE, yEv);
+    Src<SRC>::eval(k, u[0].x, q.p * q.ir, u[2].y, yE, yEv);
   }
   return pk::pair(yE, yEv);
 }
@@ -162,7 +162,7 @@ __device__ __forceinline__ void hll3(const P<float>& k, f2 (&L)[NP], f2 (&R)[NP]
 // Limited slopes of one pair of fields from its one-sided differences.
 template <int LIM>
 __device__ __forceinline__ f2 slope2(f2 a, f2 b) {
-  return pk::pair(limit<LIM, float>(a.x, b.x), limit<LIM, float>(a.y, b.y));
+  return pk::pair(limit<LIM>(a.x, b.x), limit<LIM>(a.y, b.y));
 }
 
 // Shared memory: sU[NP][TY+2][TX+2] (plane q with the second ring), sW and sF
@@ -396,7 +396,7 @@ stepnd3f_kernel(const KParams kp, float* __restrict__ bufA, float* __restrict__ 
       } else {
         const Pr3 qn = prim3<PP>(k, un);
         const float v2 = fmaf(qn.vyz.y, qn.vyz.y, fmaf(qn.vyz.x, qn.vyz.x, qn.vx * qn.vx));
-        cfl_cell<float, PP, SRC>(k, un[0].x, qn.kin2, speed_of<float>(v2), un[2].x, un[2].y,
+        cfl_cell<PP, SRC>(k, un[0].x, qn.kin2, speed_of(v2), un[2].x, un[2].y,
                                  smax, akey, flags);
       }
     }

@@ -476,7 +476,7 @@ cudaError_t pair_by_kind(const KParams& kp, void* a, void* b, Ctl* ctl, const in
 // (1000 x 700 cells), the issue slots being shared beyond one block.
 MarchShape stepnd_pair_shape() {
   using G = PairCfg<2>;
-  return {G::TX - 2, 0, 2, G::MINB, {1.0, 1.3, 2.0}, G::SEG};
+  return {G::TX - 2, 0, 2, 2.0, G::MINB, {1.0, 1.3, 2.0}, G::SEG};
 }
 
 // n == nullptr: set the kernels' shared-memory limits (host side, at set-up).

@@ -60,44 +60,45 @@ cudaError_t set_target_launch(int precision, Ctl* ctl, double t_end, const KPara
 template <typename R, int PP>
 __global__ void __launch_bounds__(NTU) dt_reduce_kernel(const KParams kp, const R* a, const R* b,
                                                         Ctl* ctl, int dim, int64_t ncell) {
+  __shared__ float s_word;
+  if (threadIdx.x == 0) s_word = 0.0f;
+  __syncthreads();
   const R* U = vload(&ctl->cur) ? b : a;
   const P<R> k(kp);
-  R smax = 0, akey = -INFINITY;
-  uint32_t flags = 0;
-  if constexpr (PP == 3) {        // perturbation layout
-    for (int64_t i = (int64_t)blockIdx.x * NTU + threadIdx.x; i < ncell;
-         i += (int64_t)gridDim.x * NTU) {
-      if (dim == 1) {
-        const R u[4] = {U[i], U[ncell + i], U[2 * ncell + i], U[3 * ncell + i]};
-        cell_bound<R, 3, 1>(k, u, smax, akey, flags);
-      } else if (dim == 2) {
-        float u[5];
-        for (int f = 0; f < 5; ++f) u[f] = U[f * ncell + i];
-        psn::bound<2, 1>(k, u, smax, akey, flags);
-      } else {
-        float u[6];
-        for (int f = 0; f < 6; ++f) u[f] = U[f * ncell + i];
-        psn::bound<3, 1>(k, u, smax, akey, flags);
-      }
-    }
-    reduce_and_finalize<R, NTU>(ctl, kp, smax, akey, flags, false);
-    return;
-  }
+  Acc<R> acc(&s_word);
   for (int64_t i = (int64_t)blockIdx.x * NTU + threadIdx.x; i < ncell;
        i += (int64_t)gridDim.x * NTU) {
-    const R rho = U[i];
-    const R ir = Ar<R>::rcp(rho);
-    R kin2 = 0, v2 = 0;
-    for (int d = 0; d < dim; ++d) {
-      const R m = U[(1 + d) * ncell + i], v = m * ir;
-      kin2 += m * v;
-      v2 += v * v;
+    if constexpr (PP == 3 || std::is_same<R, double>::value) {
+      // the perturbation layout, and double
+      if (dim == 1) {
+        const R u[4] = {U[i], U[ncell + i], U[2 * ncell + i], U[3 * ncell + i]};
+        cell_bound<PP, 1>(k, u, acc);
+      } else if (dim == 2) {
+        R u[5];
+        for (int f = 0; f < 5; ++f) u[f] = U[f * ncell + i];
+        if constexpr (PP == 3) psn::bound<2, 1>(k, u, acc.smax, acc.akey, acc.flags);
+        else d64::bound<2, 1>(k, u, acc);
+      } else {
+        R u[6];
+        for (int f = 0; f < 6; ++f) u[f] = U[f * ncell + i];
+        if constexpr (PP == 3) psn::bound<3, 1>(k, u, acc.smax, acc.akey, acc.flags);
+        else d64::bound<3, 1>(k, u, acc);
+      }
+    } else {
+      const R rho = U[i];
+      const R ir = Ar<R>::rcp(rho);
+      R kin2 = 0, v2 = 0;
+      for (int d = 0; d < dim; ++d) {
+        const R m = U[(1 + d) * ncell + i], v = m * ir;
+        kin2 += m * v;
+        v2 += v * v;
+      }
+      const R vmag = dim == 1 ? fabsf(U[ncell + i] * ir) : speed_of(v2);
+      cfl_cell<PP, 1>(k, rho, kin2, vmag, U[(1 + dim) * ncell + i], U[(2 + dim) * ncell + i],
+                      acc.smax, acc.akey, acc.flags);
     }
-    const R vmag = dim == 1 ? fabs(U[ncell + i] * ir) : speed_of<R>(v2);
-    cfl_cell<R, PP, 1>(k, rho, kin2, vmag, U[(1 + dim) * ncell + i], U[(2 + dim) * ncell + i],
-                       smax, akey, flags);
   }
-  reduce_and_finalize<R, NTU>(ctl, kp, smax, akey, flags, false);
+  reduce_and_finalize<R, NTU>(ctl, kp, acc.smax, acc.akey, acc.flags, false);
 }
 
 static int grid_small(int64_t count) {

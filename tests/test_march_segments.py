@@ -20,7 +20,7 @@ def rule(tmp_path_factory):
     src.write_text("""#include "sv_march.h"
 extern "C" int segs(int cx, int cy, int step, int occ, int dim, int64_t nx, int64_t ny, int64_t nz,
                     int64_t cap, int sms) {
-  const sv::MarchShape g = {cx, cy, step, occ, {1.0, 1.3, 2.0}, 0};
+  const sv::MarchShape g = {cx, cy, step, 2.0, occ, {1.0, 1.3, 2.0}, 0};
   const int64_t n[3] = {nx, ny, nz};
   return sv::march_segments(g, dim, n, cap, sms);
 }""")
