@@ -168,16 +168,17 @@ int sv_step(sv_solver* s, int64_t nsteps);
 /* How the steps of a solver are launched (sv_set_launch).
    SV_LAUNCH_PER_STEP: one kernel launch per step (two for SV_HEUN), replayed
      from a CUDA graph of 32 steps.
-   SV_LAUNCH_PERSISTENT: 1D MUSCL-Hancock only -- one cooperative launch runs
-     up to 65536 steps, its blocks resident throughout; the block that
-     finishes a step last computes the next dt and releases the others (a
-     grid-wide barrier).  Bitwise the same results as per-step launches.
-     Every barrier wait gives up after about 2 s with SV_FLAG_STALL, which
-     sv_run_to reports as SV_ESTALL.
+   SV_LAUNCH_PERSISTENT: 1D MUSCL-Hancock only -- one launch runs up to 65536
+     steps, its blocks resident throughout, exchanging cells and dt bounds
+     after every step.  Bitwise the same results as per-step launches.
+     Every wait gives up after about 2 s with SV_FLAG_STALL, which sv_run_to
+     reports as SV_ESTALL.
    SV_LAUNCH_AUTO (default): persistent for 1D MUSCL-Hancock grids of at most
-     one 64-cell chunk per two SMs (4864 cells on a GB300), where a step is
-     short enough for the gap between launches to matter; per-step launches
-     otherwise. */
+     one 64-cell chunk per two SMs (4864 cells on a GB300).  On larger 1D grids
+     single float steps are per-step launches, and so are all steps of grids that
+     do not fit in the device's registers (182400 cells in float, 34048 in double
+     on a GB300); runs of several steps on grids that do fit go through the
+     resident launches too. */
 #define SV_LAUNCH_AUTO       0
 #define SV_LAUNCH_PER_STEP   1
 #define SV_LAUNCH_PERSISTENT 2
@@ -187,7 +188,7 @@ int sv_step(sv_solver* s, int64_t nsteps);
    or no cooperative launch on the device).  Takes effect at the next step. */
 int sv_set_launch(sv_solver* s, int mode);
 
-/* The mode the next steps will use (SV_LAUNCH_PER_STEP or
+/* The mode a single next step will use (SV_LAUNCH_PER_STEP or
    SV_LAUNCH_PERSISTENT; AUTO resolved). */
 int sv_get_launch(sv_solver* s, int* mode);
 

@@ -52,6 +52,9 @@ struct sv_solver {
   std::vector<SolverConfig> cfgs;      // launch configurations of the per-step kernel
   int config = 0;                      // current index into cfgs
   int loop_grid = 0;                   // persistent 1D loop: blocks (0 = not available)
+  ResShape res = {0, 0, 0};            // resident 1D loop (blocks 0: grid too large for it)
+  uint64_t* res_words = nullptr;       // its exchange words
+  uint32_t res_epoch = 0;              // its launches so far
   bool loop_fits = false;              // ... at most one 64-cell chunk per SM
   int launch = SV_LAUNCH_AUTO;
   cudaGraphExec_t graph = nullptr;
@@ -67,7 +70,7 @@ constexpr int64_t kLoopChunk = 1 << 16;   // steps per persistent launch at most
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Layout {
-  size_t state, staging, ctl, partial, sums, total;
+  size_t state, staging, ctl, partial, sums, words, total;
 };
 
 int check_inputs(const sv_params* p, const sv_grid* g) {
@@ -119,7 +122,8 @@ Layout layout(const sv_params* p, const sv_grid* g) {
   L.ctl = align_up(sizeof(Ctl));
   L.partial = align_up((size_t)sums_blocks() * (size_t)nf * 2 * 8);
   L.sums = align_up(8 * 8);
-  L.total = 2 * L.state + L.staging + L.ctl + L.partial + L.sums;
+  L.words = g->dim == 1 && p->method == SV_HANCOCK ? align_up(res1d_word_bytes(p->precision, ncell)) : 0;
+  L.total = 2 * L.state + L.staging + L.ctl + L.partial + L.sums + L.words;
   return L;
 }
 
@@ -172,14 +176,23 @@ int ensure_graph(sv_solver* s) {
   return SV_OK;
 }
 
-// The persistent loop serves 1D MUSCL-Hancock solvers: always when asked for,
-// by default on grids of at most one 64-cell chunk per two SMs, where a step
-// is short enough for the gap between launches to matter (measured on a
-// GB300 with the float finalize: 7.8 instead of 10.1 us per float step at 200
-// cells, equal at 1600-5000 cells, 25-33% slower from 2e4 cells on).
+// The persistent modes serve 1D MUSCL-Hancock solvers: always when asked for,
+// by default on grids of at most one 64-cell chunk per two SMs.  They run the
+// resident loop, or, on grids it does not hold, the sliding-warp loop
+// (sv_loop1d.cu).
 bool use_loop(const sv_solver* s) {
   if (s->loop_grid < 1) return false;
   return s->launch == SV_LAUNCH_PERSISTENT || (s->launch == SV_LAUNCH_AUTO && s->loop_fits);
+}
+
+// Whether a run of n steps goes through the resident loop: in the persistent
+// modes, and in AUTO mode on any grid it holds, for runs of at least two steps
+// in float (10^5 cells: one step 10.8 us here, 10.0 per step; two 14.6 and
+// 20.2) and for any run in double (2 x 10^4 cells: one step 21 and 51 us).
+bool use_resident(const sv_solver* s, int64_t n) {
+  if (s->res.blocks < 1) return false;
+  return use_loop(s) ||
+         (s->launch == SV_LAUNCH_AUTO && n >= (s->p.precision == SV_FP64 ? 1 : 2));
 }
 
 // Launch configurations a solver can choose from, the default first.
@@ -250,6 +263,15 @@ int apply_config(sv_solver* s, int idx) {
 
 int issue_steps(sv_solver* s, int64_t n) {
   if (n <= 0) return SV_OK;
+  if (use_resident(s, n)) {
+    while (n > 0) {
+      const int64_t m = n < kLoopChunk ? n : kLoopChunk;
+      SV_TRY(res1d_launch(s->p.precision, s->kp, s->buf[0], s->buf[1], s->ctl, s->res_words,
+                          s->ncell, s->res, (int)m, ++s->res_epoch, s->stream));
+      n -= m;
+    }
+    return SV_OK;
+  }
   if (use_loop(s)) {
     while (n > 0) {
       const int64_t m = n < kLoopChunk ? n : kLoopChunk;
@@ -419,6 +441,7 @@ int sv_init(const sv_params* p, const sv_grid* g, void* cuda_stream, void* devic
   s->ctl = (Ctl*)(m + 2 * L.state + L.staging);
   s->partial = (double*)(m + 2 * L.state + L.staging + L.ctl);
   s->sums_out = (double*)(m + 2 * L.state + L.staging + L.ctl + L.partial);
+  s->res_words = (uint64_t*)(m + 2 * L.state + L.staging + L.ctl + L.partial + L.sums);
 
   rc = SV_OK;
   if (cudaMallocHost((void**)&s->host_ctl, sizeof(Ctl)) != cudaSuccess ||
@@ -441,6 +464,8 @@ int sv_init(const sv_params* p, const sv_grid* g, void* cuda_stream, void* devic
     s->loop_grid = loop1d_grid(s->kp, p->precision, s->ncell, &cap);
     if (cudaGetDevice(&dev) == cudaSuccess)
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    s->res = res1d_shape(s->kp, p->precision, s->ncell);
+    if (L.words && cudaMemsetAsync(s->res_words, 0, L.words, s->stream) != cudaSuccess) rc = SV_ECUDA;
     s->loop_fits = s->loop_grid > 0 && 2 * ((s->ncell + 63) / 64) <= (int64_t)sms;
   }
   if (rc == SV_OK) {
@@ -510,8 +535,8 @@ int sv_run_to(sv_solver* s, double t_end, int64_t max_steps, int64_t* steps_take
     if (!(est >= 1.0)) est = 1.0;
     int64_t n = est > 1e15 ? (int64_t)1e15 : (int64_t)est;
     n = n > 4096 ? 4096 : n;
-    // the persistent loop stops by itself at t_end: no estimate needed
-    if (use_loop(s)) n = kLoopChunk;
+    // the persistent loops stop by themselves at t_end: no estimate needed
+    if (use_loop(s) || use_resident(s, n)) n = kLoopChunk;
     if (n > max_steps - done) n = max_steps - done;
     if (n < 1) n = 1;
     rc = issue_steps(s, n);

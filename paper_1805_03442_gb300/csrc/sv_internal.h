@@ -51,6 +51,28 @@ int loop1d_grid(const KParams& kp, int precision, int64_t N, int* cap);
 cudaError_t loop1d_launch(int precision, const KParams& kp, void* a, void* b, Ctl* ctl, int64_t N,
                           int grid, int64_t nmax, cudaStream_t st);
 
+// 1D steps with the state resident in registers (sv_res1d.cu).  Blocks of up to
+// kResWarps* warps (the register file at 102 / 255 registers a thread; float
+// 182400 cells, double 34048 on 152 SMs), at most one per SM and kResBlocks in
+// all.  A grid of at most kResLone* warps runs in one block, without the
+// exchange through L2 (0.6 us of a step); a larger one in blocks of at least
+// kResFew* warps: fewer warps leave schedulers idle, more share them.  Float, us
+// per step by warps per block: 1000 cells 2.50 (2) 2.21 (4) 2.35 (8) 2.75 (all
+// 17); 20000 cells 3.09 (4) 3.21 (8) 3.51 (16).  Double: 1600 cells 9.49 (2, 3)
+// 9.95 (4) 16.1 (8: two warps per FP64 unit).
+constexpr int kResBlocks = 160;
+constexpr int kResWarpsF = 20, kResWarpsD = 8;
+constexpr int kResLoneF = 12, kResLoneD = 4;
+constexpr int kResFewF = 4, kResFewD = 3;
+struct ResShape {
+  int blocks, threads, wtot;    // blocks 0: not available for this grid
+};
+ResShape res1d_shape(const KParams& kp, int precision, int64_t N);
+size_t res1d_word_bytes(int precision, int64_t N);   // exchange words, zeroed once
+cudaError_t res1d_launch(int precision, const KParams& kp, void* a, void* b, Ctl* ctl,
+                         uint64_t* words, int64_t N, const ResShape& r, int nmax, uint32_t epoch,
+                         cudaStream_t st);
+
 // 1D Heun (SSP-RK2) stages (sv_heun1d.cu); stage 1 or 2
 int heun1d_grid(const KParams& kp, int precision);
 cudaError_t heun1d_launch(int precision, int stage, const KParams& kp, void* a, void* b, Ctl* ctl,

@@ -26,7 +26,7 @@ namespace sv {
 struct KParams {
   double gamma, g1, Ck, Q0, tau0, inv_tau0;
   double tau_rho, tau_T, Q_rho, Q_T, I_rho, I_T;
-  double h, cfl, c_tau;
+  double h, inv_h, cfl, cfl_h, c_tau;   // inv_h = 1 / h, cfl_h = cfl h
   int limiter;   // 0 minmod, 1 van Leer, 2 MC
   int frozen;    // 1: no source at all (Q = I = 0, 1/tau = 0)
   int qi_zero;   // 1: all Q and I exponents are zero (Q = I = Q0)
@@ -73,6 +73,8 @@ inline void kparams_finish(KParams& k) {
   k.f[13] = (float)(-k.tau_rho);
   k.f[14] = (float)(-k.tau_T);
   k.f[15] = (float)(k.g1 - (double)k.f[1]);
+  k.inv_h = 1.0 / k.h;
+  k.cfl_h = k.cfl * k.h;
   k.fdt[0] = (float)(k.cfl * k.h);
   k.fdt[1] = (float)(1.0 / k.h);
   k.fdt[2] = (float)(0.5 / k.h);
@@ -259,22 +261,25 @@ __device__ __forceinline__ StepCtl block_step_ctl(const Ctl* ctl) {
 }
 
 // The dt-derived factors of the next step in the kernel's arithmetic type.
-// Float solvers form them in float from the float dt (a product by the
-// stored 1/h and 1/(2h): no FP64 divide on the step's serial path).
+// Products by the stored 1/h and 1/(2h) (no divide on the step's serial path),
+// in float from the float dt for float solvers.
 template <typename R> struct StepDt;
 template <> struct StepDt<double> {
   double dt, dtdx, dt_2h, dt_2;
   __device__ __forceinline__ explicit StepDt(const StepCtl& c)
       : dt(c.dt), dtdx(c.dtdx), dt_2h(c.dt_2h), dt_2(c.dt_2) {}
   __device__ __forceinline__ StepDt(double d, const KParams& kp)
-      : dt(d), dtdx(d / kp.h), dt_2h(d / (2.0 * kp.h)), dt_2(0.5 * d) {}
+      : dt(d), dtdx(d * kp.inv_h), dt_2h(d * (0.5 * kp.inv_h)), dt_2(0.5 * d) {}
+  __device__ __forceinline__ StepDt(const KParams& kp, double d) : StepDt(d, kp) {}
 };
 template <> struct StepDt<float> {
   float dt, dtdx, dt_2h, dt_2;
   __device__ __forceinline__ explicit StepDt(const StepCtl& c)
       : dt(c.fdt), dtdx(c.fdtdx), dt_2h(c.fdt_2h), dt_2(c.fdt_2) {}
   __device__ __forceinline__ StepDt(double d, const KParams& kp)
-      : dt((float)d), dtdx(dt * kp.fdt[1]), dt_2h(dt * kp.fdt[2]), dt_2(0.5f * dt) {}
+      : StepDt(kp, (float)d) {}
+  __device__ __forceinline__ StepDt(const KParams& kp, float d)
+      : dt(d), dtdx(d * kp.fdt[1]), dt_2h(d * kp.fdt[2]), dt_2(0.5f * d) {}
 };
 
 // ---------------------------------------------------------------- eq. 5

@@ -65,9 +65,9 @@ __device__ __forceinline__ void cfl_cell(const P<float>& k, float rho, float kin
 // per step evaluates it on the step's serial path, in the solver's own type:
 // float solvers stay off the narrow FP64 pipe, whose divide and exp2 take
 // microseconds of latency on one thread.
-__device__ __forceinline__ double dt_from_maxima(const KParams& kp, double smax, double akey,
-                                                 uint32_t& flags) {
-  double dt = kp.cfl * kp.h / smax;
+__device__ __forceinline__ double step_rule(const KParams& kp, double smax, double akey,
+                                            uint32_t& flags) {
+  double dt = d64::mul(kp.cfl_h, d64::rcp(smax));
   if (!kp.frozen) {
     const double cap = kp.c_tau * -akey;          // akey = -min tau
     if (cap < dt) dt = cap;
@@ -75,15 +75,20 @@ __device__ __forceinline__ double dt_from_maxima(const KParams& kp, double smax,
   if (!(dt > 0.0) || !isfinite(dt)) flags |= FLAG_DT;
   return dt;
 }
-__device__ __forceinline__ double dt_from_maxima(const KParams& kp, float smax, float akey,
-                                                 uint32_t& flags) {
+__device__ __forceinline__ float step_rule(const KParams& kp, float smax, float akey,
+                                           uint32_t& flags) {
   float dt = __fdiv_rn(kp.fdt[0], smax);
   if (!kp.frozen) {
     const float cap = kp.fdt[3] * Ar<float>::ex2(-akey);   // c_tau tau0 2^-a = c_tau min tau
     if (cap < dt) dt = cap;
   }
   if (!(dt > 0.0f) || !isfinite(dt)) flags |= FLAG_DT;
-  return (double)dt;
+  return dt;
+}
+template <typename R>
+__device__ __forceinline__ double dt_from_maxima(const KParams& kp, R smax, R akey,
+                                                 uint32_t& flags) {
+  return (double)step_rule(kp, smax, akey, flags);
 }
 
 // Store the next step's dt and its derived factors (StepDt of the solver's
