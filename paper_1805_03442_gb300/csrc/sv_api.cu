@@ -54,7 +54,6 @@ struct sv_solver {
   int loop_grid = 0;                   // persistent 1D loop: blocks (0 = not available)
   ResShape res = {0, 0, 0};            // resident 1D loop (blocks 0: grid too large for it)
   uint64_t* res_words = nullptr;       // its exchange words
-  uint32_t res_epoch = 0;              // its launches so far
   bool loop_fits = false;              // ... at most one 64-cell chunk per SM
   int launch = SV_LAUNCH_AUTO;
   cudaGraphExec_t graph = nullptr;
@@ -267,7 +266,7 @@ int issue_steps(sv_solver* s, int64_t n) {
     while (n > 0) {
       const int64_t m = n < kLoopChunk ? n : kLoopChunk;
       SV_TRY(res1d_launch(s->p.precision, s->kp, s->buf[0], s->buf[1], s->ctl, s->res_words,
-                          s->ncell, s->res, (int)m, ++s->res_epoch, s->stream));
+                          s->ncell, s->res, (int)m, s->stream));
       n -= m;
     }
     return SV_OK;

@@ -70,7 +70,7 @@ struct ResShape {
 ResShape res1d_shape(const KParams& kp, int precision, int64_t N);
 size_t res1d_word_bytes(int precision, int64_t N);   // exchange words, zeroed once
 cudaError_t res1d_launch(int precision, const KParams& kp, void* a, void* b, Ctl* ctl,
-                         uint64_t* words, int64_t N, const ResShape& r, int nmax, uint32_t epoch,
+                         uint64_t* words, int64_t N, const ResShape& r, int nmax,
                          cudaStream_t st);
 
 // 1D Heun (SSP-RK2) stages (sv_heun1d.cu); stage 1 or 2

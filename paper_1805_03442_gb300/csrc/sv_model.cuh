@@ -129,7 +129,7 @@ struct Ctl {
   uint32_t ticket;     // blocks finished in the running launch
   uint64_t smax_key;   // order-preserving key of max signal speed
   uint64_t tau_key;    // order-preserving key of the tau bound (see finalize)
-  uint32_t gen;        // grid-barrier generation of the persistent step loop
+  uint32_t gen;        // generation of the persistent loops (barriers; resident launches)
   uint32_t pad32;
   double pad[3];
 };

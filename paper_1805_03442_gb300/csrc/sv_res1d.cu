@@ -57,12 +57,11 @@ ResShape res1d_shape(const KParams& kp, int precision, int64_t N) {
 }
 
 cudaError_t res1d_launch(int precision, const KParams& kp, void* a, void* b, Ctl* ctl,
-                         uint64_t* words, int64_t N, const ResShape& r, int nmax, uint32_t epoch,
+                         uint64_t* words, int64_t N, const ResShape& r, int nmax,
                          cudaStream_t st) {
   if (r.blocks < 1 || nmax < 1 || nmax > 65536) return cudaErrorInvalidValue;
   int n32 = (int)N, wtot = r.wtot;
-  epoch &= 0x3fffu;
-  void* args[] = {(void*)&kp, &a, &b, &ctl, &words, &n32, &wtot, &nmax, &epoch};
+  void* args[] = {(void*)&kp, &a, &b, &ctl, &words, &n32, &wtot, &nmax};
   if (r.blocks == 1)
     return cudaLaunchKernel(pick(kp, precision), dim3(1), dim3(r.threads), args, 0, st);
   return cudaLaunchCooperativeKernel(pick(kp, precision), dim3(r.blocks), dim3(r.threads), args, 0,

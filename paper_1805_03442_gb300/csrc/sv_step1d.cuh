@@ -194,13 +194,26 @@ __device__ __forceinline__ void update_cell(const P<R>& k, const R (&u)[4], cons
   if (CFL) cell_bound<PP, SRC>(k, un, m);
 }
 
-// State of the driven boundary's ghost cell centred at x at time t (double).
+// State of the driven boundary's ghost cell centred at x at time t (double):
+// the envelope and k x of the cell, the wave's phase, and one field of it.
+struct DriveCell {
+  double env, kx;
+  __device__ __forceinline__ DriveCell(const KParams& kp, double x)
+      : env(exp(d64::mul(-kp.drv_kim, x))), kx(d64::mul(kp.drv_kre, x)) {}
+  __device__ __forceinline__ void phase(const KParams& kp, double t, double& s, double& c) const {
+    sincos(d64::fma(-kp.drv_omega, t, kx), &s, &c);
+  }
+  __device__ __forceinline__ double field(double base, double re, double im, double s,
+                                          double c) const {
+    return d64::fma(env, d64::fma(re, c, -d64::mul(im, s)), base);
+  }
+};
 __device__ __forceinline__ void drive_state(const KParams& kp, double x, double t, double (&u)[4]) {
-  const double env = exp(-kp.drv_kim * x);
+  const DriveCell d(kp, x);
   double s, c;
-  sincos(kp.drv_kre * x - kp.drv_omega * t, &s, &c);
+  d.phase(kp, t, s, c);
 #pragma unroll
-  for (int f = 0; f < 4; ++f) u[f] = kp.drv_base[f] + env * (kp.drv_are[f] * c - kp.drv_aim[f] * s);
+  for (int f = 0; f < 4; ++f) u[f] = d.field(kp.drv_base[f], kp.drv_are[f], kp.drv_aim[f], s, c);
 }
 
 // One warp's share of a step: chunks [c0, c1) (64 cells each) of the periodic

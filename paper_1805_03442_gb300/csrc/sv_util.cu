@@ -19,6 +19,7 @@ __global__ void ctl_reset_kernel(Ctl* ctl, double t) {
   ctl->last = 0;
   ctl->flags = 0;
   ctl->ticket = 0;
+  ctl->gen += 1u;      // words of a resident launch that stalled are not the next one's
   ctl->smax_key = key_of(0.0);
   ctl->tau_key = key_of(-INFINITY);
 }

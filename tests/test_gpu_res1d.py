@@ -88,3 +88,31 @@ def test_stops_when_a_cell_fails(sv):
     r = pair(sv, sv.Params(precision=sv.FP32, tau0=0.2), N, U0,
              lambda s: s.run_to(0.05, check=False)[0])
     assert r[3] != 0 and r[5] in (sv.SV_ENONPHYS, sv.SV_EDT)
+
+
+def test_captured_run_replays(sv):
+    """A run captured in a CUDA graph and replayed: every replay is a launch
+    of its own to the exchange words."""
+    torch = pytest.importorskip("torch")
+    N = 20000
+    P = sv.Params(precision=sv.FP32, tau0=0.3)
+    U0 = inputs.random_states(1, N, seed=1, smooth=True)
+    st = torch.cuda.Stream()
+    with sv.Solver(P, (N,), (1.0,), stream=st) as s:
+        s.write_state(U0)
+        s.step(3)
+        s.write_state(U0)
+        st.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=st):
+            s.step(3)
+        for _ in range(8):
+            g.replay()
+        torch.cuda.synchronize()
+        U, t = s.read_state()
+    with sv.Solver(P, (N,), (1.0,)) as r:
+        r.set_launch(sv.LAUNCH_PER_STEP)
+        r.write_state(U0)
+        r.step(24)
+        V, tr = r.read_state()
+    assert t == tr and np.array_equal(U, V)
