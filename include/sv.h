@@ -329,9 +329,11 @@ int sv_batch_mode_log(sv_batch* b, int64_t run, double* t, double* re, double* i
 
 void sv_batch_free(sv_batch* b);
 
-/* Launch configurations of a batch: the block size per run, 256 (default) or
-   128 threads.  Same results, different speed: smaller blocks keep more runs
-   in flight and idle fewer warps on small runs.  Set before sv_batch_run. */
+/* Launch configurations of a batch: the block size, 256 (default) or 128
+   threads.  Same results, different speed: smaller blocks keep more runs
+   in flight and idle fewer warps on small runs.  Set before sv_batch_run.
+   The library steps each run on one block, or on a cluster of 2 to 16 when
+   there are too few runs to fill the device. */
 int sv_batch_num_configs(sv_batch* b, int* count);
 int sv_batch_set_config(sv_batch* b, int index);
 int sv_batch_get_config(sv_batch* b, int* index, char* desc, size_t cap);

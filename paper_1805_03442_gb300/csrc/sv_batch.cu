@@ -2,14 +2,16 @@
 // periodic runs of uneven sizes and parameters advanced to their own t_end by
 // ONE persistent launch.
 //
-// Each CTA takes a run from a device work queue (the runs of >= 8192 cells
-// first, largest first, then the others by decreasing estimated cost,
-// n^2 t_end / L, so that the longest runs start first), steps it
-// to completion with the same per-warp MUSCL-Hancock body as the single-grid
-// kernel (sv_step1d.cuh), and only then takes the next run.  A run's dt
-// reduction is CTA-local (shared memory + __syncthreads): there is no grid
-// barrier and no host round trip per step.  At sampled times the CTA
-// projects the velocity on the logged Fourier mode m,
+// A cluster of blocks (one block when there are runs enough to fill the device)
+// takes a run from a device work queue (the runs of >= 8192 cells first, largest
+// first, then the others by decreasing estimated cost, n^2 t_end / L, so that the
+// longest runs start first), steps it to completion with the window arithmetic
+// of the resident loop (sv_window1d.cuh), and only then takes the next run.  A
+// run whose windows fit one per warp keeps its state in registers; a longer one
+// streams its windows through L2.  The dt reduction goes through the cluster's
+// shared memory with one barrier per step: no grid barrier, no host round trip.
+// At sampled times the cluster projects the velocity on the logged Fourier mode
+// m,
 //   a_m(t) = (1/n) sum_j v_j exp(-i 2 pi m (j + 1/2) / n),
 // which is what a growth-rate fit of the linear stage needs.
 #include <math.h>
@@ -19,6 +21,7 @@
 #include <algorithm>
 #include <new>
 #include <numeric>
+#include <queue>
 #include <vector>
 
 #include "sv_batch_kernel.cuh"
@@ -46,10 +49,18 @@ struct sv_batch {
   int* order = nullptr;
   int* queue = nullptr;
   double* logs = nullptr;
-  std::vector<RunDev> host_runs;
+  std::vector<RunDev> host_runs;      // the records as last uploaded
+  // Page-locked copies of what a run leaves: its records and logs, copied behind
+  // the kernel as part of the run, and room for one run's state.  Null (the
+  // reads then copy from the device each time) beyond kMirrorBytes.
+  RunDev* mirror = nullptr;
+  double* mirror_logs = nullptr;
+  unsigned char* staging = nullptr;
   std::vector<int64_t> n;
+  std::vector<int> host_order;        // queue order
   int64_t total_elems = 0;
-  int grid = 0;
+  int grid = 0;                       // blocks: a multiple of `cluster`
+  int cluster = 1;                    // blocks per run
   int nt = 256;                       // threads per run (block size)
   int config = 0;                     // index into kBatchConfigs
   void* fn = nullptr;
@@ -62,9 +73,18 @@ namespace {
 constexpr size_t kAlignB = 256;
 size_t alb(size_t x) { return (x + kAlignB - 1) / kAlignB * kAlignB; }
 
+constexpr size_t kMirrorBytes = (size_t)64 << 20;
+
 struct BLayout {
   size_t state, runs, order, queue, logs, total;
 };
+
+// What a step costs besides its rounds of windows, in rounds (1.4 us with the
+// device full), for clusters of 1, 2, 4, 8 and 16 blocks: a run that streams its
+// windows, and one that keeps its single round in registers.  Measured, us per
+// step with every SM full, streaming 2 rounds / resident: 3.86 / 2.16 (1 block),
+// 4.29 / 2.40 (2), 4.34 / 2.42 (4), 4.36 / 2.77 (8), 4.59 / 3.08 (16).
+constexpr double kBatchLat[5][2] = {{0.8, 0.55}, {1.0, 0.7}, {1.05, 0.73}, {1.1, 0.95}, {1.2, 1.2}};
 
 // Runs of at least this many cells lead the queue (sv_batch_init).
 constexpr int64_t kBigRun = 8192;
@@ -105,27 +125,27 @@ BLayout blayout(const sv_params* p, const sv_run* r, int64_t nruns, int log_cap)
     if (e_ != cudaSuccess) return SV_ECUDA;  \
   } while (0)
 
-int upload(sv_batch* b, const double* host) {
-  // host: concatenation over runs of (4, n_r) field-major blocks
-  const size_t es = (size_t)b->esize;
-  std::vector<unsigned char> tmp((size_t)b->total_elems * es, 0);
-  int64_t src = 0;
+// The runs' states in the device's format and layout (host: concatenation over
+// runs of (4, n_r) field-major blocks; the perturbation layout holds U - ref,
+// the difference taken in double).
+template <typename R>
+void pack_states(const sv_batch* b, const double* host, R* out) {
   for (int64_t i = 0; i < b->nruns; ++i) {
-    const int64_t n = b->n[i], st = stride_of(n), off = b->host_runs[i].off;
-    const double* ref = b->host_runs[i].kp.ref;
-    for (int f = 0; f < 4; ++f)
-      for (int64_t j = 0; j < n; ++j) {
-        // the perturbation layout holds U - ref (difference in double)
-        const double v = host[src + f * n + j] - (b->ps ? ref[f] : 0.0);
-        const size_t at = (size_t)(off + f * st + j);
-        if (es == 8) memcpy(&tmp[at * 8], &v, 8);
-        else {
-          const float fv = (float)v;
-          memcpy(&tmp[at * 4], &fv, 4);
-        }
-      }
-    src += 4 * n;
+    const int64_t n = b->n[(size_t)i], st = stride_of(n);
+    const RunDev& r = b->host_runs[(size_t)i];
+    for (int f = 0; f < 4; ++f) {
+      const double ref = b->ps ? r.kp.ref[f] : 0.0;
+      R* o = out + r.off + f * st;
+      for (int64_t j = 0; j < n; ++j) o[j] = (R)(host[j] - ref);
+      host += n;
+    }
   }
+}
+
+int upload(sv_batch* b, const double* host) {
+  std::vector<unsigned char> tmp((size_t)b->total_elems * (size_t)b->esize, 0);
+  if (b->esize == 8) pack_states(b, host, (double*)tmp.data());
+  else pack_states(b, host, (float*)tmp.data());
   SVB_TRY(cudaMemcpyAsync(b->buf[0], tmp.data(), tmp.size(), cudaMemcpyHostToDevice, b->stream));
   for (auto& r : b->host_runs) {
     r.t = 0.0;
@@ -136,7 +156,9 @@ int upload(sv_batch* b, const double* host) {
   }
   SVB_TRY(cudaMemcpyAsync(b->runs, b->host_runs.data(), sizeof(RunDev) * b->host_runs.size(),
                           cudaMemcpyHostToDevice, b->stream));
-  return cudaStreamSynchronize(b->stream) == cudaSuccess ? SV_OK : SV_ECUDA;
+  if (cudaStreamSynchronize(b->stream) != cudaSuccess) return SV_ECUDA;
+  if (b->mirror) memcpy(b->mirror, b->host_runs.data(), sizeof(RunDev) * b->host_runs.size());
+  return SV_OK;
 }
 
 // Launch configurations of the batch kernel (sv_batch_set_config): block size
@@ -152,24 +174,89 @@ constexpr BatchConfig kBatchConfigs[] = {
 };
 constexpr int kNumBatchConfigs = (int)(sizeof(kBatchConfigs) / sizeof(kBatchConfigs[0]));
 
-size_t batch_smem(int precision, int nt) {
-  return (size_t)(nt / 32) * (precision == SV_FP64 ? ring1d_bytes<double>() : ring1d_bytes<float>());
+// The launch of `clusters` clusters of C blocks.
+struct BatchLaunch {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  BatchLaunch(int clusters, int C, int nt, cudaStream_t st) {
+    cfg.gridDim = dim3((unsigned)(clusters * C));
+    cfg.blockDim = dim3((unsigned)nt);
+    cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)C;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = C > 1 ? 1 : 0;
+  }
+};
+
+// Time of the whole sweep, in rounds, when runs are taken in queue order by
+// `groups` groups of `warps` warps each: a step is the rounds of windows its
+// busiest warp does and `lat`, the number of steps is estimated by the frozen
+// sound speed at rest.
+double sweep_time(const sv_batch* b, const std::vector<int>& order, int groups, int warps,
+                  const double (&lat)[2]) {
+  const int own = b->esize == 8 ? 28 : 60;
+  std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
+  for (int i = 0; i < groups && i < (int)order.size(); ++i) free_at.push(0.0);
+  double end = 0.0;
+  for (int id : order) {
+    const RunDev& r = b->host_runs[(size_t)id];
+    const int64_t windows = (r.n + own - 1) / own;
+    const double rounds = (double)((windows + warps - 1) / warps);
+    const double steps = std::max(1.0, std::min((double)b->max_steps,
+                                                r.t_end * sqrt(r.kp.gamma) / r.kp.cfl_h));
+    const double t = free_at.top() + steps * (rounds + lat[rounds == 1.0 ? 1 : 0]);
+    free_at.pop();
+    free_at.push(t);
+    if (t > end) end = t;
+  }
+  return end;
 }
 
-// Pick the kernel of configuration c, set its shared-memory limit and the
-// persistent grid (host side, outside any capture).
+// Pick the kernel of configuration c, the blocks per run and the persistent
+// grid (host side, outside any capture).
+//
+// One block per run keeps the device busiest when there are many more runs than
+// blocks fit; with fewer, or when a few long runs are left at the end, SMs
+// idle while the others step one run each, so a run is given a cluster of 2 to
+// 16 blocks, whichever ends the sweep first by sweep_time.  Sweeps in ms, one
+// block of a sliding kernel per run (before) / one block / this choice: 256 runs
+// of 256-6000 cells 67 / 63 / 17.9 (8 blocks), 400 of 500-4000 38 / 32 / 12.4 (4),
+// 2000 of 256-2000 13.1 / 9.2 / 9.2 (1), 8 of 20000-40000 168 / 178 / 17.1 (16).
 int apply_config(sv_batch* b, int c) {
   const int nt = kBatchConfigs[c].nt;
   void* fn = nt == 128 ? batch_pick128(b->p.limiter, b->p.precision)
                        : batch_pick256(b->p.limiter, b->p.precision);
   int dev = 0, sms = 0, per = 0;
-  const size_t smem = batch_smem(b->p.precision, nt);
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-          cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, nt, smem) != cudaSuccess)
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, nt, 0) != cudaSuccess)
     return SV_ECUDA;
+  int groups = sms * (per < 1 ? 1 : per), cluster = 1;
+  double best = sweep_time(b, b->host_order, groups, nt / 32, kBatchLat[0]);
+  // 16 blocks are beyond the size every device supports: asked for, and skipped
+  // below where it is not available
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+    cudaGetLastError();
+  for (int C = 2, i = 1; C <= kBatchCluster; C *= 2, ++i) {
+    int nc = 0;
+    const BatchLaunch l(1, C, nt, nullptr);
+    if (cudaOccupancyMaxActiveClusters(&nc, fn, &l.cfg) != cudaSuccess) {
+      cudaGetLastError();
+      continue;
+    }
+    // clusters of 16: half of what the occupancy query says run at once (18
+    // asked for: 5.8 us per step, 9: 3.1)
+    if (C == 16) nc /= 2;
+    if (nc < 1) continue;
+    const double t = sweep_time(b, b->host_order, nc, C * nt / 32, kBatchLat[i]);
+    if (t < best) {
+      best = t;
+      groups = nc;
+      cluster = C;
+    }
+  }
   if (b->graph) {
     if (cudaStreamSynchronize(b->stream) != cudaSuccess) return SV_ECUDA;
     cudaGraphExecDestroy(b->graph);
@@ -178,9 +265,14 @@ int apply_config(sv_batch* b, int c) {
   b->fn = fn;
   b->nt = nt;
   b->config = c;
-  b->grid = sms * (per < 1 ? 1 : per);
-  if ((int64_t)b->grid > b->nruns) b->grid = (int)b->nruns;
+  b->cluster = cluster;
+  if ((int64_t)groups > b->nruns) groups = (int)b->nruns;
+  b->grid = groups * cluster;
   return SV_OK;
+}
+
+size_t log_bytes(const sv_batch* b) {
+  return sizeof(double) * 3 * (size_t)b->log_cap * (size_t)b->nruns;
 }
 
 cudaError_t launch_batch(sv_batch* b, cudaStream_t st) {
@@ -189,16 +281,31 @@ cudaError_t launch_batch(sv_batch* b, cudaStream_t st) {
   int nr = (int)b->nruns;
   int lc = b->log_cap;
   int64_t ms = b->max_steps;
-  void* args[] = {&b->runs, &b->order, &nr, &b->queue, &b->buf[0], &b->buf[1], &b->logs, &lc, &ms};
-  return cudaLaunchKernel(b->fn, dim3(b->grid), dim3(b->nt), args, batch_smem(b->p.precision, b->nt),
-                          st);
+  void* args[] = {&b->runs, &b->order, &nr, &b->queue, &b->buf[0], &b->buf[1], &b->logs, &lc, &ms,
+                  &b->cluster};
+  const BatchLaunch l(b->grid / b->cluster, b->cluster, b->nt, st);
+  e = cudaLaunchKernelExC(&l.cfg, b->fn, args);
+  if (e == cudaSuccess && b->mirror)
+    e = cudaMemcpyAsync(b->mirror, b->runs, sizeof(RunDev) * (size_t)b->nruns,
+                        cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess && b->mirror_logs)
+    e = cudaMemcpyAsync(b->mirror_logs, b->logs, log_bytes(b), cudaMemcpyDeviceToHost, st);
+  return e;
 }
 
-int read_runs(sv_batch* b) {
-  SVB_TRY(cudaMemcpyAsync(b->host_runs.data(), b->runs, sizeof(RunDev) * b->host_runs.size(),
-                          cudaMemcpyDeviceToHost, b->stream));
+// Record of a run, once the stream's work is done.
+int read_run(sv_batch* b, int64_t run, RunDev& d) {
+  if (!b->mirror)
+    SVB_TRY(cudaMemcpyAsync(&d, b->runs + run, sizeof(RunDev), cudaMemcpyDeviceToHost, b->stream));
   SVB_TRY(cudaStreamSynchronize(b->stream));
+  if (b->mirror) d = b->mirror[run];
   return SV_OK;
+}
+
+template <typename R>
+void unpack_state(const R* src, int64_t n, int64_t st, const double* ref, double* out) {
+  for (int f = 0; f < 4; ++f)
+    for (int64_t j = 0; j < n; ++j) out[f * n + j] = (ref ? ref[f] : 0.0) + (double)src[f * st + j];
 }
 
 }  // namespace
@@ -306,11 +413,29 @@ int sv_batch_init(const sv_params* p, const sv_run* runs, int64_t nruns,
     return big(a) ? runs[a].n > runs[c].n : cost[a] > cost[c];
   });
 
+  b->host_order = order;
   rc = SV_OK;
   if (cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking) != cudaSuccess ||
       cudaMemcpyAsync(b->order, order.data(), sizeof(int) * order.size(), cudaMemcpyHostToDevice,
                       b->stream) != cudaSuccess)
     rc = SV_ECUDA;
+  {
+    // page-locked copies where they are of a size to keep; without them the
+    // reads copy from the device
+    int64_t widest = 0;
+    for (int64_t n : b->n) widest = std::max(widest, 4 * stride_of(n) * (int64_t)b->esize);
+    const size_t rec = sizeof(RunDev) * (size_t)nruns;
+    auto lock = [](void** p, size_t bytes) {
+      if (bytes == 0 || bytes > kMirrorBytes) return;
+      if (cudaMallocHost(p, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        *p = nullptr;
+      }
+    };
+    lock((void**)&b->mirror, rec);
+    if (b->mirror) lock((void**)&b->mirror_logs, log_bytes(b));
+    lock((void**)&b->staging, (size_t)widest);
+  }
   if (rc == SV_OK) rc = apply_config(b, 0);
   if (rc == SV_OK) rc = upload(b, host_states);
   if (rc != SV_OK) {
@@ -357,29 +482,25 @@ int sv_batch_sync(sv_batch* b) {
 int sv_batch_read(sv_batch* b, int64_t run, double* host_soa, double* t, int64_t* steps,
                   uint32_t* flags) {
   if (!b || run < 0 || run >= b->nruns) return SV_EINVAL;
-  int rc = read_runs(b);
+  RunDev d;
+  int rc = read_run(b, run, d);
   if (rc != SV_OK) return rc;
-  const RunDev& d = b->host_runs[(size_t)run];
   if (t) *t = d.t;
   if (steps) *steps = d.steps;
   if (flags) *flags = d.flags;
   if (host_soa) {
     const int64_t n = d.n, st = d.stride;
     const size_t es = (size_t)b->esize;
-    std::vector<unsigned char> tmp((size_t)(4 * st) * es);
+    const size_t bytes = (size_t)(4 * st) * es;
+    std::vector<unsigned char> pageable;
+    if (!b->staging) pageable.resize(bytes);
+    unsigned char* const tmp = b->staging ? b->staging : pageable.data();
     const char* src = (const char*)b->buf[d.cur ? 1 : 0] + (size_t)d.off * es;
-    SVB_TRY(cudaMemcpyAsync(tmp.data(), src, tmp.size(), cudaMemcpyDeviceToHost, b->stream));
+    SVB_TRY(cudaMemcpyAsync(tmp, src, bytes, cudaMemcpyDeviceToHost, b->stream));
     SVB_TRY(cudaStreamSynchronize(b->stream));
-    for (int f = 0; f < 4; ++f)
-      for (int64_t j = 0; j < n; ++j) {
-        const size_t at = (size_t)(f * st + j);
-        if (es == 8) memcpy(&host_soa[f * n + j], &tmp[at * 8], 8);
-        else {
-          float fv;
-          memcpy(&fv, &tmp[at * 4], 4);
-          host_soa[f * n + j] = (b->ps ? d.kp.ref[f] : 0.0) + (double)fv;
-        }
-      }
+    const double* ref = b->ps ? d.kp.ref : nullptr;
+    if (es == 8) unpack_state((const double*)tmp, n, st, ref, host_soa);
+    else unpack_state((const float*)tmp, n, st, ref, host_soa);
   }
   return SV_OK;
 }
@@ -387,15 +508,22 @@ int sv_batch_read(sv_batch* b, int64_t run, double* host_soa, double* t, int64_t
 int sv_batch_mode_log(sv_batch* b, int64_t run, double* t, double* re, double* im, int64_t cap,
                       int64_t* count) {
   if (!b || run < 0 || run >= b->nruns || cap < 0) return SV_EINVAL;
-  int rc = read_runs(b);
+  RunDev d;
+  int rc = read_run(b, run, d);
   if (rc != SV_OK) return rc;
-  const int64_t c = std::min<int64_t>(b->host_runs[(size_t)run].log_count, cap);
+  const int64_t c = std::min<int64_t>(d.log_count, cap);
   if (count) *count = c;
   if (c > 0) {
-    std::vector<double> tmp((size_t)c * 3);
-    SVB_TRY(cudaMemcpyAsync(tmp.data(), b->logs + run * (int64_t)b->log_cap * 3,
-                            sizeof(double) * tmp.size(), cudaMemcpyDeviceToHost, b->stream));
-    SVB_TRY(cudaStreamSynchronize(b->stream));
+    const int64_t at = run * (int64_t)b->log_cap * 3;
+    std::vector<double> copy;
+    const double* tmp = b->mirror_logs + at;
+    if (!b->mirror_logs) {
+      copy.resize((size_t)c * 3);
+      SVB_TRY(cudaMemcpyAsync(copy.data(), b->logs + at, sizeof(double) * copy.size(),
+                              cudaMemcpyDeviceToHost, b->stream));
+      SVB_TRY(cudaStreamSynchronize(b->stream));
+      tmp = copy.data();
+    }
     for (int64_t i = 0; i < c; ++i) {
       if (t) t[i] = tmp[(size_t)(3 * i)];
       if (re) re[i] = tmp[(size_t)(3 * i + 1)];
@@ -431,6 +559,9 @@ void sv_batch_free(sv_batch* b) {
   if (b->stream || b->mem) cudaStreamSynchronize(b->stream);
   if (b->graph) cudaGraphExecDestroy(b->graph);
   if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
+  if (b->mirror) cudaFreeHost(b->mirror);
+  if (b->mirror_logs) cudaFreeHost(b->mirror_logs);
+  if (b->staging) cudaFreeHost(b->staging);
   if (b->owns_mem && b->mem) cudaFree(b->mem);
   delete b;
 }

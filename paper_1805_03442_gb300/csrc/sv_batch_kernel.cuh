@@ -5,7 +5,7 @@
 
 #include "sv.h"
 #include "sv_internal.h"
-#include "sv_step1d.cuh"
+#include "sv_window1d.cuh"
 
 namespace sv {
 
@@ -21,205 +21,360 @@ struct RunDev {
 
 constexpr uint32_t FLAG_MAXSTEPS = SV_FLAG_MAXSTEPS;
 
-template <int NT, typename R>
-__device__ __forceinline__ void block_max(R& smax, R& akey, uint32_t& flags, R* s_a, R* s_b,
-                                          uint32_t* s_f) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    smax = fmax(smax, __shfl_xor_sync(0xffffffffu, smax, o));
-    akey = fmax(akey, __shfl_xor_sync(0xffffffffu, akey, o));
-    flags |= __shfl_xor_sync(0xffffffffu, flags, o);
-  }
-  const int w = threadIdx.x >> 5;
-  if ((threadIdx.x & 31) == 0) {
-    s_a[w] = smax;
-    s_b[w] = akey;
-    s_f[w] = flags;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0)
-    for (int i = 1; i < NT / 32; ++i) {
-      smax = fmax(smax, s_a[i]);
-      akey = fmax(akey, s_b[i]);
-      flags |= s_f[i];
-    }
+// A run is stepped by a cluster of C blocks (1 <= C <= kBatchCluster).
+constexpr int kBatchCluster = 16;
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// Barrier of the run's blocks: orders their shared and global stores before
+// the loads behind it.
+__device__ __forceinline__ void cluster_bar(int C) {
+  if (C == 1) __syncthreads();
+  else
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Store a 4-byte word to the same shared variable of block `rank`.
+__device__ __forceinline__ void put_cluster(const void* var, int rank, uint32_t v) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(var);
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(r), "r"(v) : "memory");
+}
+__device__ __forceinline__ void put_cluster(const float* var, int rank, float v) {
+  put_cluster((const void*)var, rank, __float_as_uint(v));
+}
+__device__ __forceinline__ void put_cluster(const double* var, int rank, double v) {
+  put_cluster((const void*)var, rank, (uint32_t)__double2loint(v));
+  put_cluster((const char*)var + 4, rank, (uint32_t)__double2hiint(v));
 }
 
-template <int NT, typename R>
-__device__ __forceinline__ void block_sum2(R& a, R& b, R* s_a, R* s_b) {
+template <typename R, int W>
+struct BatchSmem {
+  static constexpr int NS = W * kBatchCluster;
+  KParams kp;                            // the run's parameters
+  R smax[2][NS], akey[2][NS];            // every warp of the cluster, by step parity
+  uint32_t fl[2][NS];
+  R sum[2][NS];                          // every warp's part of a logged amplitude
+  R halo[2][W][2][2][4];                 // by parity: each warp's halo cells (side, cell, field)
+  double t;
+  float word[2];                         // speed threshold of the double bound, by parity
+  int run;
+};
+
+// The cluster's maxima of what each thread has folded: every warp tells every
+// block, one barrier, every warp reads them all.
+template <typename R, int W>
+__device__ __forceinline__ void cluster_max(BatchSmem<R, W>& S, int q, int rank, int C,
+                                            const Acc<R>& acc, R& smax, R& akey, uint32_t& flags) {
+  const int lane = threadIdx.x & 31, me = rank * W + (threadIdx.x >> 5);
+  const R m = warp_max(acc.smax), a = warp_max(acc.akey);
+  const uint32_t f = __reduce_or_sync(0xffffffffu, acc.flags);
+  if (lane < C) {
+    put_cluster(&S.smax[q][me], lane, m);
+    put_cluster(&S.akey[q][me], lane, a);
+    put_cluster((const void*)&S.fl[q][me], lane, f);
+  }
+  cluster_bar(C);
+  smax = (R)0;
+  akey = (R)-INFINITY;
+  flags = 0;
+  for (int i = lane; i < C * W; i += 32) {
+    smax = fmax(smax, S.smax[q][i]);
+    akey = fmax(akey, S.akey[q][i]);
+    flags |= S.fl[q][i];
+  }
+  smax = warp_max(smax);
+  akey = warp_max(akey);
+  flags = __reduce_or_sync(0xffffffffu, flags);
+}
+
+// The window of cells c0 - 2 .. c0 + 62 (float; double: c0 + 29) of a periodic
+// run into registers.  Through L2: neighbouring cells are other blocks' work.
+__device__ __forceinline__ void load_window(const float* U, int n, int stride, int c0,
+                                            float (&X)[2][4]) {
+  const int lane = threadIdx.x & 31, j = c0 - 2 + 2 * lane;
+  if (c0 >= 2 && c0 + 62 <= n) {               // c0 and stride are even: 8-byte loads
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    a += __shfl_xor_sync(0xffffffffu, a, o);
-    b += __shfl_xor_sync(0xffffffffu, b, o);
-  }
-  const int w = threadIdx.x >> 5;
-  if ((threadIdx.x & 31) == 0) {
-    s_a[w] = a;
-    s_b[w] = b;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0)
-    for (int i = 1; i < NT / 32; ++i) {
-      a += s_a[i];
-      b += s_b[i];
+    for (int f = 0; f < 4; ++f) {
+      const float2 v = __ldcg(reinterpret_cast<const float2*>(U + f * stride + j));
+      X[0][f] = v.x;
+      X[1][f] = v.y;
     }
+  } else {
+    const int a = wrap(j, n), b = wrap(j + 1, n);
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      X[0][f] = __ldcg(U + f * stride + a);
+      X[1][f] = __ldcg(U + f * stride + b);
+    }
+  }
+}
+__device__ __forceinline__ void load_window(const double* U, int n, int stride, int c0,
+                                            double (&X)[1][4]) {
+  const int j = c0 - 2 + (int)(threadIdx.x & 31);
+  const int a = j >= 0 && j < n ? j : wrap(j, n);
+#pragma unroll
+  for (int f = 0; f < 4; ++f) X[0][f] = __ldcg(U + f * stride + a);
+}
+__device__ __forceinline__ void store_window(float* U, int stride, int c0,
+                                             const float (&X)[2][4], const bool (&own)[2]) {
+  const int j = c0 - 2 + 2 * (int)(threadIdx.x & 31);
+#pragma unroll
+  for (int f = 0; f < 4; ++f) {
+    if (own[0] && own[1])
+      *reinterpret_cast<float2*>(U + f * stride + j) = make_float2(X[0][f], X[1][f]);
+    else if (own[0])
+      U[f * stride + j] = X[0][f];
+  }
+}
+__device__ __forceinline__ void store_window(double* U, int stride, int c0,
+                                             const double (&X)[1][4], const bool (&own)[1]) {
+  const int j = c0 - 2 + (int)(threadIdx.x & 31);
+#pragma unroll
+  for (int f = 0; f < 4; ++f)
+    if (own[0]) U[f * stride + j] = X[0][f];
+}
+
+// Step run `rd` to its end.  Every thread of the cluster follows the same
+// decisions: they all see the same maxima.
+template <typename R, int PP, int LIM, int SRC, int W>
+__device__ void batch_run(BatchSmem<R, W>& S, RunDev* rd, R* A, R* B, double* lg, int log_cap,
+                          int64_t max_steps, int rank, int C) {
+  constexpr int CPL = Win<R>::CPL, OWN = Win<R>::OWN;
+  const KParams& kp = S.kp;
+  const P<R> k(kp);
+  const int n = rd->n, stride = rd->stride, mode = rd->mode;
+  const double t_end = rd->t_end;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int gw = rank * W + w, nw = C * W;
+  const int nwin = (n + OWN - 1) / OWN;
+  // contiguous windows [w0, w1) of this warp
+  const int w0 = (int)((int64_t)gw * nwin / nw), w1 = (int)((int64_t)(gw + 1) * nwin / nw);
+  const double log_dt = log_cap > 1 ? t_end / (double)(log_cap - 1) : INFINITY;
+  const bool logs = mode > 0 && log_cap > 0;
+
+  // a_m of the current state (buffer U), a sample of the log
+  auto log_mode = [&](const R* U, double t, int slot) {
+    R re = 0, im = 0;
+    for (int j = gw * 32 + lane; j < n; j += nw * 32) {
+      const R r0 = __ldcg(U + j);
+      const R v = __ldcg(U + stride + j) / (PP == 3 ? (R)1 + r0 : r0);   // PP 3: perturbations
+      R sn, cs;
+      const R ph = (R)(2.0 * mode) * ((R)j + (R)0.5) / (R)n;
+      if constexpr (sizeof(R) == 4) sincospif(ph, &sn, &cs);
+      else sincospi(ph, &sn, &cs);
+      re += v * cs;
+      im -= v * sn;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      re += __shfl_xor_sync(0xffffffffu, re, o);
+      im += __shfl_xor_sync(0xffffffffu, im, o);
+    }
+    if (lane == 0) {
+      put_cluster(&S.sum[0][gw], 0, re);
+      put_cluster(&S.sum[1][gw], 0, im);
+    }
+    cluster_bar(C);
+    if (rank == 0 && threadIdx.x == 0) {
+      R a = 0, b = 0;
+      for (int i = 0; i < nw; ++i) {
+        a += S.sum[0][i];
+        b += S.sum[1][i];
+      }
+      lg[3 * slot + 0] = t;
+      lg[3 * slot + 1] = (double)a / n;
+      lg[3 * slot + 2] = (double)b / n;
+    }
+    cluster_bar(C);                    // the sums have been read
+  };
+
+  // dt of the initial state (same per-cell bound as every step)
+  Clock<R> ck;
+  int log_count = 0;
+  double next_log = INFINITY;
+  {
+    Acc<R> acc(&S.word[0]);
+    for (int j = gw * 32 + lane; j < n; j += nw * 32) {
+      const R u[4] = {A[j], A[stride + j], A[2 * stride + j], A[3 * stride + j]};
+      cell_bound<PP, 1>(k, u, acc);
+    }
+    R smax, akey;
+    uint32_t flags;
+    cluster_max<R, W>(S, 0, rank, C, acc, smax, akey, flags);
+    const R d = step_rule(kp, smax, akey, flags);
+    const double t = rd->t, r = t_end - t;
+    const bool go = flags == 0 && t < t_end;
+    const bool last = go && (double)d >= r;
+    ck.start(t, t_end, last ? (R)r : d, last);
+    ck.flags = flags;
+    ck.stop = !go;
+    if (logs) {
+      log_mode(A, t, 0);
+      log_count = 1;
+      next_log = t + log_dt;
+      if (log_count < log_cap) ck.due(next_log);
+    }
+  }
+  uint32_t cur = 0;
+  int64_t steps = 0;
+  // the step with these maxima is complete: the clock, and a log sample of
+  // the state that `state()` provides in global memory
+  auto finish = [&](R smax, R akey, uint32_t flags, auto&& state) {
+    ++steps;
+    const bool exact =
+        ck.advance(kp, smax, akey, flags, w == 0, &S.t, steps >= max_steps, [&](double t) {
+          return steps >= max_steps && t < t_end ? FLAG_MAXSTEPS : 0u;
+        });
+    if (exact && logs && log_count < log_cap && (ck.t >= next_log || ck.stop)) {
+      log_mode(state(), ck.t, log_count);
+      ++log_count;
+      while (next_log <= ck.t) next_log += log_dt;
+    }
+    if (exact && !ck.stop && logs) ck.due(log_count < log_cap ? next_log : t_end);
+  };
+  if (nwin <= nw && n >= 2) {
+    // one window per warp: the state stays in registers, neighbours' cells come
+    // through shared memory with the maxima's barrier, and global memory (A) is
+    // written for the log samples and at the end only
+    const bool live = gw < nwin;
+    const int c0 = live ? (int)((int64_t)gw * n / nwin) : 0;
+    const int cnt = live ? (int)((int64_t)(gw + 1) * n / nwin) - c0 : 0;
+    const int lg_w = gw == 0 ? nwin - 1 : gw - 1, rg_w = gw == nwin - 1 ? 0 : gw + 1;
+    R X[CPL][4];
+    bool own[CPL];
+#pragma unroll
+    for (int c = 0; c < CPL; ++c) {
+      const int pos = CPL * lane + c;
+      own[c] = live && pos >= 2 && pos < 2 + cnt;
+      const int j = wrap(c0 - 2 + (pos < cnt + 3 ? pos : cnt + 3), n);
+#pragma unroll
+      for (int f = 0; f < 4; ++f) X[c][f] = A[f * stride + j];
+    }
+    auto save = [&]() -> const R* {
+#pragma unroll
+      for (int c = 0; c < CPL; ++c)
+        if (own[c])
+#pragma unroll
+          for (int f = 0; f < 4; ++f) A[f * stride + c0 - 2 + CPL * lane + c] = X[c][f];
+      return A;
+    };
+    if (!ck.stop) cluster_bar(C);        // every warp has read its cells of A
+    while (!ck.stop) {
+      const int q = (int)(steps + 1) & 1;
+      const StepDt<R> sd(kp, ck.dt);
+      if (threadIdx.x == 0) S.word[q ^ 1] = 0.0f;   // as in the resident loop
+      Acc<R> acc(&S.word[q]);
+      if (live) window_step<PP, LIM, SRC>(k, X, own, sd, acc);
+#pragma unroll
+      for (int c = 0; c < CPL; ++c) {
+        const int pos = CPL * lane + c, pf = pos - 2, pl = pos - cnt;
+        if (own[c] && pf < 2)            // the left neighbour's right halo
+#pragma unroll
+          for (int f = 0; f < 4; ++f)
+            put_cluster(&S.halo[q][lg_w % W][1][pf][f], lg_w / W, X[c][f]);
+        if (own[c] && pl >= 0)           // the right neighbour's left halo
+#pragma unroll
+          for (int f = 0; f < 4; ++f)
+            put_cluster(&S.halo[q][rg_w % W][0][pl][f], rg_w / W, X[c][f]);
+      }
+      R smax, akey;
+      uint32_t flags;
+      cluster_max<R, W>(S, q, rank, C, acc, smax, akey, flags);
+#pragma unroll
+      for (int c = 0; c < CPL; ++c) {
+        const int pos = CPL * lane + c, rh = pos - (2 + cnt);
+        if (live && (pos < 2 || rh == 0 || rh == 1))
+#pragma unroll
+          for (int f = 0; f < 4; ++f)
+            X[c][f] = pos < 2 ? S.halo[q][w][0][pos][f] : S.halo[q][w][1][rh][f];
+      }
+      finish(smax, akey, flags, [&]() -> const R* {
+        const R* a = save();
+        cluster_bar(C);
+        return a;
+      });
+    }
+    save();
+  } else {
+    while (!ck.stop) {
+      const int q = (int)(steps + 1) & 1;
+      const StepDt<R> sd(kp, ck.dt);
+      const R* Uin = cur ? B : A;
+      R* Uout = cur ? A : B;
+      if (threadIdx.x == 0) S.word[q ^ 1] = 0.0f;   // as in the resident loop
+      Acc<R> acc(&S.word[q]);
+      R X[CPL][4], Y[CPL][4];
+      if (w0 < w1) load_window(Uin, n, stride, w0 * OWN, Y);
+      for (int i = w0; i < w1; ++i) {
+        const int c0 = i * OWN, cnt = min(OWN, n - c0);
+        bool own[CPL];
+#pragma unroll
+        for (int c = 0; c < CPL; ++c) {
+          const int pos = CPL * lane + c;
+          own[c] = pos >= 2 && pos < 2 + cnt;
+#pragma unroll
+          for (int f = 0; f < 4; ++f) X[c][f] = Y[c][f];
+        }
+        if (i + 1 < w1) load_window(Uin, n, stride, c0 + OWN, Y);   // in flight meanwhile
+        window_step<PP, LIM, SRC>(k, X, own, sd, acc);
+        store_window(Uout, stride, c0, X, own);
+      }
+      R smax, akey;
+      uint32_t flags;
+      cluster_max<R, W>(S, q, rank, C, acc, smax, akey, flags);   // orders the stores too
+      cur ^= 1u;
+      finish(smax, akey, flags, [&]() -> const R* { return cur ? B : A; });
+    }
+  }
+  if (rank == 0 && threadIdx.x == 0) {
+    rd->t = ck.t;
+    rd->steps = steps;
+    rd->flags = ck.flags;
+    rd->cur = cur;
+    rd->log_count = log_count;
+  }
 }
 
 // Every run is stepped with the source variant a single 1D solver with the
 // same parameters would use (none in the frozen limit, pump = sink for zero
 // exponents, general otherwise), chosen per run at run time, so that a batched
-// run and a looped solver run execute the same instructions.
+// run and a looped solver run execute the same operations.
 template <typename R, int PP, int LIM, int NTB, int MINB>
 __global__ void __launch_bounds__(NTB, MINB)
 batch_kernel(RunDev* __restrict__ runs, const int* __restrict__ order, int nruns,
-             int* __restrict__ queue, R* __restrict__ bufA, R* __restrict__ bufB,
-             double* __restrict__ logs, int log_cap, int64_t max_steps) {
-  __shared__ R s_a[NTB / 32], s_b[NTB / 32];
-  __shared__ uint32_t s_f[NTB / 32];
-  __shared__ int s_run, s_stop, s_last, s_log;
-  __shared__ double s_dt, s_t;
-  __shared__ float s_word;              // speed threshold of the double bound (d64::Bound)
-  __shared__ R s_step[4];               // dt, dt/h, dt/(2h), dt/2 of the next step
-  extern __shared__ __align__(16) unsigned char smemb[];   // per-warp rings
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  R* ring = reinterpret_cast<R*>(smemb) + warp * (ring1d_bytes<R>() / sizeof(R));
-
+             int* __restrict__ queue, R* bufA, R* bufB, double* logs, int log_cap,
+             int64_t max_steps, int C) {
+  constexpr int W = NTB / 32;
+  __shared__ BatchSmem<R, W> S;
+  const int rank = C == 1 ? 0 : (int)cluster_rank();
+  cluster_bar(C);                      // every block of the cluster has started
   for (;;) {
-    if (threadIdx.x == 0) {
-      s_run = atomicAdd(queue, 1);
-      s_word = 0.0f;
+    if (rank == 0 && threadIdx.x < 32) {
+      int r = 0;
+      if (threadIdx.x == 0) r = atomicAdd(queue, 1);
+      r = __shfl_sync(0xffffffffu, r, 0);
+      if ((int)threadIdx.x < C) put_cluster((const void*)&S.run, (int)threadIdx.x, (uint32_t)r);
     }
-    __syncthreads();
-    const int qi = s_run;
+    cluster_bar(C);
+    const int qi = S.run;
     if (qi >= nruns) break;
-    RunDev* rd = runs + order[qi];
-    const KParams& kp = rd->kp;
-    const P<R> k(kp);
-    const int n = rd->n, stride = rd->stride, mode = rd->mode, src = rd->src;
-    const double t_end = rd->t_end;
-    R* A = bufA + rd->off;
-    R* B = bufB + rd->off;
-    const int nchunk = (n + 63) / 64;
-    const int c0 = warp * nchunk / (NTB / 32), c1 = (warp + 1) * nchunk / (NTB / 32);
-    double* lg = logs + (int64_t)(order[qi]) * log_cap * 3;
-    const double log_dt = log_cap > 1 ? t_end / (double)(log_cap - 1) : INFINITY;
-
-    // logging of a_m at the current state (buffer U)
-    auto log_mode = [&](const R* U, double t, int slot) {
-      R re = 0, im = 0;
-      for (int j = threadIdx.x; j < n; j += NTB) {
-        const R v = U[stride + j] / (PP == 3 ? (R)1 + U[j] : U[j]);   // PP 3: perturbations
-        R sn, cs;
-        const R ph = (R)(2.0 * mode) * ((R)j + (R)0.5) / (R)n;
-        if constexpr (sizeof(R) == 4) sincospif(ph, &sn, &cs);
-        else sincospi(ph, &sn, &cs);
-        re += v * cs;
-        im -= v * sn;
-      }
-      block_sum2<NTB>(re, im, s_a, s_b);
-      if (threadIdx.x == 0) {
-        lg[3 * slot + 0] = t;
-        lg[3 * slot + 1] = (double)re / n;
-        lg[3 * slot + 2] = (double)im / n;
-      }
-      __syncthreads();
-    };
-
-    // dt of the initial state (same per-cell bound as every step)
-    {
-      Acc<R> acc(&s_word);
-      for (int j = threadIdx.x; j < n; j += NTB) {
-        const R u[4] = {A[j], A[stride + j], A[2 * stride + j], A[3 * stride + j]};
-        cell_bound<PP, 1>(k, u, acc);
-      }
-      block_max<NTB>(acc.smax, acc.akey, acc.flags, s_a, s_b, s_f);
-      if (threadIdx.x == 0) {
-        s_word = 0.0f;
-        uint32_t flags = acc.flags;
-        const double dt = dt_from_maxima(kp, acc.smax, acc.akey, flags);
-        double t = rd->t;
-        rd->flags = flags;
-        s_t = t;
-        s_stop = flags != 0 || !(t < t_end);
-        s_last = 0;
-        s_dt = dt;
-        if (!s_stop && dt >= t_end - t) {
-          s_dt = t_end - t;
-          s_last = 1;
-        }
-        const StepDt<R> sd(s_dt, kp);
-        s_step[0] = sd.dt;
-        s_step[1] = sd.dtdx;
-        s_step[2] = sd.dt_2h;
-        s_step[3] = sd.dt_2;
-      }
-      __syncthreads();
-    }
-    int log_count = 0;
-    double next_log = s_t;
-    if (mode > 0 && log_cap > 0) {
-      log_mode(A, s_t, 0);
-      log_count = 1;
-      next_log = s_t + log_dt;
-    }
-    uint32_t cur = 0;
-    int64_t steps = 0;
-    while (!s_stop) {
-      const double dtd = s_dt;
-      const R dt = s_step[0], dtdx = s_step[1], dt_2h = s_step[2], dt_2 = s_step[3];
-      const R* Uin = cur ? B : A;
-      R* Uout = cur ? A : B;
-      Acc<R> acc(&s_word);
-      if (src == 0)
-        step1d_warp<R, PP, LIM, 0>(k, Uin, Uout, n, stride, c0, c1, lane, dt, dtdx, dt_2h, dt_2,
-                                   acc, ring, kp, s_t);
-      else if (src == 1)
-        step1d_warp<R, PP, LIM, 1>(k, Uin, Uout, n, stride, c0, c1, lane, dt, dtdx, dt_2h, dt_2,
-                                   acc, ring, kp, s_t);
-      else
-        step1d_warp<R, PP, LIM, 2>(k, Uin, Uout, n, stride, c0, c1, lane, dt, dtdx, dt_2h, dt_2,
-                                   acc, ring, kp, s_t);
-      // the barrier inside block_max also orders this step's stores before the
-      // next step's loads of neighbouring warps' cells
-      block_max<NTB>(acc.smax, acc.akey, acc.flags, s_a, s_b, s_f);
-      cur ^= 1u;
-      ++steps;
-      if (threadIdx.x == 0) {
-        s_word = 0.0f;
-        uint32_t flags = acc.flags;
-        const double dt_next = dt_from_maxima(kp, acc.smax, acc.akey, flags);
-        const double t = s_last ? t_end : s_t + dtd;
-        s_t = t;
-        if (steps >= max_steps && t < t_end) flags |= FLAG_MAXSTEPS;
-        rd->flags = flags;
-        s_stop = flags != 0 || !(t < t_end);
-        s_last = 0;
-        s_dt = dt_next;
-        if (!s_stop && dt_next >= t_end - t) {
-          s_dt = t_end - t;
-          s_last = 1;
-        }
-        const StepDt<R> sd(s_dt, kp);
-        s_step[0] = sd.dt;
-        s_step[1] = sd.dtdx;
-        s_step[2] = sd.dt_2h;
-        s_step[3] = sd.dt_2;
-        s_log = mode > 0 && log_count < log_cap && (t >= next_log || s_stop);
-      }
-      __syncthreads();
-      if (s_log) {
-        log_mode(cur ? B : A, s_t, log_count);
-        ++log_count;
-        while (next_log <= s_t) next_log += log_dt;
-      }
-    }
-    if (threadIdx.x == 0) {
-      rd->t = s_t;
-      rd->steps = steps;
-      rd->cur = cur;
-      rd->log_count = log_count;
-    }
+    const int id = order[qi];
+    RunDev* rd = runs + id;
+    for (int i = threadIdx.x; i < (int)(sizeof(KParams) / 4); i += NTB)
+      reinterpret_cast<uint32_t*>(&S.kp)[i] = reinterpret_cast<const uint32_t*>(&rd->kp)[i];
+    if (threadIdx.x == 0) S.word[0] = S.word[1] = 0.0f;
     __syncthreads();
+    R* const A = bufA + rd->off;
+    R* const B = bufB + rd->off;
+    double* const lg = logs + (int64_t)id * log_cap * 3;
+    if (rd->src == 0) batch_run<R, PP, LIM, 0, W>(S, rd, A, B, lg, log_cap, max_steps, rank, C);
+    else if (rd->src == 1) batch_run<R, PP, LIM, 1, W>(S, rd, A, B, lg, log_cap, max_steps, rank, C);
+    else batch_run<R, PP, LIM, 2, W>(S, rd, A, B, lg, log_cap, max_steps, rank, C);
+    cluster_bar(C);                    // the run's record and this block's memory are free
   }
 }
 

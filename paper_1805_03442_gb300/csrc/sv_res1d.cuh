@@ -39,7 +39,7 @@
 #pragma once
 
 #include "sv_internal.h"
-#include "sv_step1d.cuh"
+#include "sv_window1d.cuh"
 
 namespace sv {
 
@@ -48,9 +48,9 @@ namespace {
 constexpr uint64_t kResStallNs = 2000000000ull;   // give up a wait after 2 s
 constexpr uint32_t kResStallIters = 1u << 24;      // ... or after this many polls
 
-template <typename R> struct Win;
-template <> struct Win<float> { static constexpr int CPL = 2, MAXW = kResWarpsF; };
-template <> struct Win<double> { static constexpr int CPL = 1, MAXW = kResWarpsD; };
+template <typename R> struct ResWarps;
+template <> struct ResWarps<float> { static constexpr int N = kResWarpsF; };
+template <> struct ResWarps<double> { static constexpr int N = kResWarpsD; };
 
 __device__ __forceinline__ void put_word(uint64_t* p, uint32_t tag, uint32_t v) {
   const uint64_t w = ((uint64_t)tag << 32) | v;
@@ -105,24 +105,6 @@ __device__ __forceinline__ bool wait_words(const uint64_t* p, bool need, uint32_
   return false;
 }
 
-// Maxima over a warp as unsigned keys (one redux instruction per 32 bits).
-__device__ __forceinline__ uint32_t fkey(float x) {
-  const uint32_t b = __float_as_uint(x);
-  return (b >> 31) ? ~b : (b | 0x80000000u);
-}
-__device__ __forceinline__ float fkey_value(uint32_t k) {
-  return __uint_as_float((k >> 31) ? (k & 0x7fffffffu) : ~k);
-}
-__device__ __forceinline__ float warp_max(float x) {
-  return fkey_value(__reduce_max_sync(0xffffffffu, fkey(x)));
-}
-__device__ __forceinline__ double warp_max(double x) {
-  const uint64_t k = key_of(x);
-  const uint32_t hi = __reduce_max_sync(0xffffffffu, (uint32_t)(k >> 32));
-  const uint32_t lo = __reduce_max_sync(0xffffffffu, (uint32_t)(k >> 32) == hi ? (uint32_t)k : 0u);
-  return key_to_double(((uint64_t)hi << 32) | lo);
-}
-
 __device__ __forceinline__ uint32_t word_of(float x, int) { return __float_as_uint(x); }
 __device__ __forceinline__ uint32_t word_of(double x, int i) {
   return i ? (uint32_t)__double2hiint(x) : (uint32_t)__double2loint(x);
@@ -131,66 +113,6 @@ __device__ __forceinline__ void from_words(const uint32_t* w, float& x) { x = __
 __device__ __forceinline__ void from_words(const uint32_t* w, double& x) {
   x = __hiloint2double((int)w[1], (int)w[0]);
 }
-
-// Step size of the run, advanced by every warp alike.  The time itself is kept
-// by one warp (`keep`), whose sums nothing waits for: an FP64 operation takes
-// a scheduler 64 cycles.  The others hold a float below t_end - t, which says
-// that a step cannot be the last one; when it does not, all warps take the time
-// from shared memory and decide exactly, as the per-step finalize does.
-template <typename R>
-struct Clock {
-  double t, t_end;                // t: in the keeping warp
-  R dt, dt_cfl;                   // of the next step; before the clamp to t_end
-  float rest, slack;              // below t_end - t; above t's rounding per step
-  uint32_t flags;
-  bool last, stop;
-  static __device__ __forceinline__ float below(double x) {
-    return (float)x * (1.0f - 0x1p-20f);
-  }
-  // The step of `dt` is complete with these maxima: the next one's dt.  Called
-  // by the whole block; `word` is shared memory.
-  __device__ __forceinline__ void advance(const KParams& kp, R smax, R akey, uint32_t f, bool keep,
-                                          volatile double* word) {
-    if (keep) t = last ? t_end : t + (double)dt;
-    const R d = step_rule(kp, smax, akey, f);
-    dt_cfl = d;
-    flags = f;
-    const float df = Clock::above(d);
-    // the roundings of this and of t stay below the two margins (t_end = inf:
-    // rest stays inf)
-    rest = fmaf(rest, 1.0f - 0x1p-21f, -(Clock::above(dt) + slack));
-    dt = d;
-    stop = f != 0;
-    if (!stop && !last && df < rest) return;
-    // near t_end, or a flag: exactly
-    if (keep && (threadIdx.x & 31) == 0) *word = t;
-    __syncthreads();
-    const double now = *word;
-    __syncthreads();
-    t = now;
-    last = false;
-    if (f || !(now < t_end)) {
-      dt = (R)0;
-      stop = true;
-    } else {
-      const double r = t_end - now;
-      rest = below(r);
-      if ((double)d >= r) {
-        dt_last = r;
-        dt = (R)r;
-        last = true;
-      }
-    }
-  }
-  double dt_last;                 // the last step's dt (t_end - t)
-  static __device__ __forceinline__ float above(float x) { return x; }
-  // the float at or above a positive double, from its bits; +inf beyond range
-  static __device__ __forceinline__ float above(double x) {
-    bool ok = true;
-    const float v = d64::trunc_f(x, ok);
-    return ok ? v * (1.0f + 0x1p-22f) : INFINITY;
-  }
-};
 
 template <typename R, int MAXW>
 struct ResSmem {
@@ -205,74 +127,14 @@ struct ResSmem {
   int stall;
 };
 
-// One step of a warp's cells (float: two per lane).  X: the lane's cells,
-// own[]: which of them are updated; folds their bounds.
-template <int PP, int LIM, int SRC>
-__device__ __forceinline__ void res_step(const P<float>& k, float (&X)[2][4], const bool (&own)[2],
-                                         const StepDt<float>& sd, Acc<float>& acc) {
-  using pk::f2;
-  const f2 dt2 = pk::splat(sd.dt), ndtdx2 = pk::splat(-sd.dtdx);
-  const f2 ndt_2h2 = pk::splat(-sd.dt_2h), dt_22 = pk::splat(sd.dt_2);
-  f2 U[4], A[4], B[4], WP[4], WM[4], YE, YEv, L[4], F[4], FR[4], Nw[4];
-  float xl[4];
-#pragma unroll
-  for (int f = 0; f < 4; ++f) {
-    U[f] = pk::pair(X[0][f], X[1][f]);
-    xl[f] = __shfl_up_sync(0xffffffffu, X[1][f], 1);
-    const float xr = __shfl_down_sync(0xffffffffu, X[0][f], 1);
-    const float c = U[f].y - U[f].x;
-    A[f] = pk::pair(U[f].x - xl[f], c);
-    B[f] = pk::pair(c, xr - U[f].y);
-  }
-  pkx::predict<PP, LIM, SRC>(k, U, A, B, ndt_2h2, dt_22, WP, WM, YE, YEv);
-#pragma unroll
-  for (int f = 0; f < 4; ++f) L[f] = pk::pair(__shfl_up_sync(0xffffffffu, WP[f].y, 1), WP[f].x);
-  pkx::hll<PP>(k, L, WM, xl, U, F);
-#pragma unroll
-  for (int f = 0; f < 4; ++f) FR[f] = pk::pair(F[f].y, __shfl_down_sync(0xffffffffu, F[f].x, 1));
-  pk::update<SRC>(U, F, FR, YE, YEv, dt2, ndtdx2, Nw);
-#pragma unroll
-  for (int f = 0; f < 4; ++f) {
-    if (own[0]) X[0][f] = Nw[f].x;
-    if (own[1]) X[1][f] = Nw[f].y;
-  }
-  pkx::cfl<PP, SRC>(k, Nw, (own[0] ? 1 : 0) | (own[1] ? 2 : 0), acc.smax, acc.akey, acc.flags);
-}
-
-// The same in double, one cell per lane.
-template <int PP, int LIM, int SRC>
-__device__ __forceinline__ void res_step(const P<double>& k, double (&X)[1][4],
-                                         const bool (&own)[1], const StepDt<double>& sd,
-                                         Acc<double>& acc) {
-  double A[4], B[4], um[4], wp[4], wm[4], yE, yEv, L[4], F[4], FR[4], un[4];
-#pragma unroll
-  for (int f = 0; f < 4; ++f) {
-    um[f] = __shfl_up_sync(0xffffffffu, X[0][f], 1);
-    B[f] = d64::sub(__shfl_down_sync(0xffffffffu, X[0][f], 1), X[0][f]);
-    A[f] = __shfl_up_sync(0xffffffffu, B[f], 1);
-  }
-  d64::predict1<LIM, SRC>(k, X[0], A, B, sd.dt_2h, sd.dt_2, wp, wm, yE, yEv);
-#pragma unroll
-  for (int f = 0; f < 4; ++f) L[f] = __shfl_up_sync(0xffffffffu, wp[f], 1);
-  hll(k, L, wm, um, X[0], F);
-#pragma unroll
-  for (int f = 0; f < 4; ++f) FR[f] = __shfl_down_sync(0xffffffffu, F[f], 1);
-  if (own[0]) {
-    d64::update1<SRC>(X[0], F, FR, yE, yEv, sd.dt, sd.dtdx, un);
-    d64::bound<1, SRC>(k, un, acc);
-#pragma unroll
-    for (int f = 0; f < 4; ++f) X[0][f] = un[f];
-  }
-}
-
 // Up to nmax steps; stops once the next dt is 0 (t_end reached or a flag
 // raised).  `words`: ResWords of the exchange (several blocks only); `wtot`:
 // warps that own cells.
 template <typename R, int PP, int LIM, int SRC>
-__global__ void __launch_bounds__(Win<R>::MAXW * 32, 1)
+__global__ void __launch_bounds__(ResWarps<R>::N * 32, 1)
 res1d_kernel(const KParams kp, R* bufA, R* bufB, Ctl* ctl, uint64_t* words, int N, int wtot,
              int nmax) {
-  constexpr int CPL = Win<R>::CPL, MAXW = Win<R>::MAXW, NW = sizeof(R) / 4;
+  constexpr int CPL = Win<R>::CPL, MAXW = ResWarps<R>::N, NW = sizeof(R) / 4;
   __shared__ ResSmem<R, MAXW> S;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int W = blockDim.x >> 5, G = gridDim.x, b = blockIdx.x;
@@ -305,16 +167,8 @@ res1d_kernel(const KParams kp, R* bufA, R* bufB, Ctl* ctl, uint64_t* words, int 
   R* const U = sc.cur ? bufB : bufA;
   const P<R> k(kp);
   Clock<R> ck;
-  const StepDt<R> sd0(sc);
-  ck.t = sc.t;
-  ck.dt = sd0.dt;
-  ck.t_end = vload(&ctl->t_end);
-  ck.last = vload(&ctl->last) != 0;
+  ck.start(sc.t, vload(&ctl->t_end), StepDt<R>(sc).dt, vload(&ctl->last) != 0);
   ck.dt_last = sc.dt;
-  ck.rest = Clock<R>::below(ck.t_end - ck.t);
-  ck.slack = isfinite(ck.t_end) ? (float)((fabs(ck.t) + fabs(ck.t_end)) * 0x1p-51) : 0.0f;
-  ck.flags = 0;
-  ck.stop = false;
   const long long nsteps0 = vload(&ctl->nsteps);
   int done = 0;
 
@@ -372,7 +226,7 @@ res1d_kernel(const KParams kp, R* bufA, R* bufB, Ctl* ctl, uint64_t* words, int 
     // barrier, and next in step s + 1, which is behind this step's
     if (threadIdx.x == 0) S.word[q ^ 1] = 0.0f;
     Acc<R> acc(&S.word[q]);
-    if (live) res_step<PP, LIM, SRC>(k, X, own, sd, acc);
+    if (live) window_step<PP, LIM, SRC>(k, X, own, sd, acc);
     // publish the first and last two cells, then the bounds
 #pragma unroll
     for (int c = 0; c < CPL; ++c) {
@@ -486,7 +340,7 @@ res1d_kernel(const KParams kp, R* bufA, R* bufB, Ctl* ctl, uint64_t* words, int 
       }
     }
     // (the clamp to t_end reads and writes S.t between barriers of its own)
-    ck.advance(kp, smax, akey, flags, w == 0, &S.t);
+    ck.advance(kp, smax, akey, flags, w == 0, &S.t, false, [](double) { return 0u; });
     done = s;
     if (ck.stop || s >= nmax) break;
 
