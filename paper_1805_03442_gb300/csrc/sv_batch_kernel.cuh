@@ -5,6 +5,7 @@
 
 #include "sv.h"
 #include "sv_internal.h"
+#include "sv_cluster.cuh"
 #include "sv_window1d.cuh"
 
 namespace sv {
@@ -24,72 +25,17 @@ constexpr uint32_t FLAG_MAXSTEPS = SV_FLAG_MAXSTEPS;
 // A run is stepped by a cluster of C blocks (1 <= C <= kBatchCluster).
 constexpr int kBatchCluster = 16;
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-// Barrier of the run's blocks: orders their shared and global stores before
-// the loads behind it.
-__device__ __forceinline__ void cluster_bar(int C) {
-  if (C == 1) __syncthreads();
-  else
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// Store a 4-byte word to the same shared variable of block `rank`.
-__device__ __forceinline__ void put_cluster(const void* var, int rank, uint32_t v) {
-  const uint32_t a = (uint32_t)__cvta_generic_to_shared(var);
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(r), "r"(v) : "memory");
-}
-__device__ __forceinline__ void put_cluster(const float* var, int rank, float v) {
-  put_cluster((const void*)var, rank, __float_as_uint(v));
-}
-__device__ __forceinline__ void put_cluster(const double* var, int rank, double v) {
-  put_cluster((const void*)var, rank, (uint32_t)__double2loint(v));
-  put_cluster((const char*)var + 4, rank, (uint32_t)__double2hiint(v));
-}
-
 template <typename R, int W>
 struct BatchSmem {
   static constexpr int NS = W * kBatchCluster;
   KParams kp;                            // the run's parameters
-  R smax[2][NS], akey[2][NS];            // every warp of the cluster, by step parity
-  uint32_t fl[2][NS];
+  ClusterMax<R, NS> mx;
   R sum[2][NS];                          // every warp's part of a logged amplitude
   R halo[2][W][2][2][4];                 // by parity: each warp's halo cells (side, cell, field)
   double t;
   float word[2];                         // speed threshold of the double bound, by parity
   int run;
 };
-
-// The cluster's maxima of what each thread has folded: every warp tells every
-// block, one barrier, every warp reads them all.
-template <typename R, int W>
-__device__ __forceinline__ void cluster_max(BatchSmem<R, W>& S, int q, int rank, int C,
-                                            const Acc<R>& acc, R& smax, R& akey, uint32_t& flags) {
-  const int lane = threadIdx.x & 31, me = rank * W + (threadIdx.x >> 5);
-  const R m = warp_max(acc.smax), a = warp_max(acc.akey);
-  const uint32_t f = __reduce_or_sync(0xffffffffu, acc.flags);
-  if (lane < C) {
-    put_cluster(&S.smax[q][me], lane, m);
-    put_cluster(&S.akey[q][me], lane, a);
-    put_cluster((const void*)&S.fl[q][me], lane, f);
-  }
-  cluster_bar(C);
-  smax = (R)0;
-  akey = (R)-INFINITY;
-  flags = 0;
-  for (int i = lane; i < C * W; i += 32) {
-    smax = fmax(smax, S.smax[q][i]);
-    akey = fmax(akey, S.akey[q][i]);
-    flags |= S.fl[q][i];
-  }
-  smax = warp_max(smax);
-  akey = warp_max(akey);
-  flags = __reduce_or_sync(0xffffffffu, flags);
-}
 
 // The window of cells c0 - 2 .. c0 + 62 (float; double: c0 + 29) of a periodic
 // run into registers.  Through L2: neighbouring cells are other blocks' work.
@@ -204,7 +150,7 @@ __device__ void batch_run(BatchSmem<R, W>& S, RunDev* rd, R* A, R* B, double* lg
     }
     R smax, akey;
     uint32_t flags;
-    cluster_max<R, W>(S, 0, rank, C, acc, smax, akey, flags);
+    cluster_max(S.mx, 0, rank, C, W, acc, smax, akey, flags);
     const R d = step_rule(kp, smax, akey, flags);
     const double t = rd->t, r = t_end - t;
     const bool go = flags == 0 && t < t_end;
@@ -283,7 +229,7 @@ __device__ void batch_run(BatchSmem<R, W>& S, RunDev* rd, R* A, R* B, double* lg
       }
       R smax, akey;
       uint32_t flags;
-      cluster_max<R, W>(S, q, rank, C, acc, smax, akey, flags);
+      cluster_max(S.mx, q, rank, C, W, acc, smax, akey, flags);
 #pragma unroll
       for (int c = 0; c < CPL; ++c) {
         const int pos = CPL * lane + c, rh = pos - (2 + cnt);
@@ -325,7 +271,7 @@ __device__ void batch_run(BatchSmem<R, W>& S, RunDev* rd, R* A, R* B, double* lg
       }
       R smax, akey;
       uint32_t flags;
-      cluster_max<R, W>(S, q, rank, C, acc, smax, akey, flags);   // orders the stores too
+      cluster_max(S.mx, q, rank, C, W, acc, smax, akey, flags);   // orders the stores too
       cur ^= 1u;
       finish(smax, akey, flags, [&]() -> const R* { return cur ? B : A; });
     }

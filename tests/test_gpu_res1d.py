@@ -116,3 +116,38 @@ def test_captured_run_replays(sv):
         r.step(24)
         V, tr = r.read_state()
     assert t == tr and np.array_equal(U, V)
+
+
+@pytest.mark.parametrize("prec", ["FP32", "FP32_P64", "FP64"])
+@pytest.mark.parametrize("n", [1, 2, 3, 60, 61, 112, 113, 720, 721, 1791, 1792, 1793, 9599, 9600, 9601])
+def test_noalloc_sizes(sv, n, prec):
+    """The allocation-free step, one launch on grids a cluster holds (9600 cells
+    in float, 1792 in double), against the solver's step."""
+    torch = pytest.importorskip("torch")
+    P = sv.Params(precision=getattr(sv, prec), tau0=0.3)
+    U0 = inputs.random_states(1, n, seed=n, smooth=n > 3)
+    with sv.Solver(P, (n,), (1.0,)) as s:
+        s.set_launch(sv.LAUNCH_PER_STEP)
+        s.write_state(U0)
+        s.step(1)
+        U, t = s.read_state()
+        flags = s.status()
+    a = torch.tensor(U0, dtype=torch.float64 if prec == "FP64" else torch.float32, device="cuda")
+    b = torch.zeros_like(a)
+    dt, fl = sv.step1d_noalloc(P, n, 1.0, a.data_ptr(), b.data_ptr())
+    assert dt == t and fl == flags
+    assert np.array_equal(b.double().cpu().numpy(), U)
+
+
+@pytest.mark.parametrize("n", [500, 20000])
+def test_noalloc_nonphysical_input(sv, n):
+    """A state whose dt cannot be formed: no step is taken, dt 0, the flags say so."""
+    torch = pytest.importorskip("torch")
+    P = sv.Params(precision=sv.FP32)
+    U0 = inputs.random_states(1, n, seed=n, smooth=True)
+    U0[0, n // 2] = -1.0
+    a = torch.tensor(U0, dtype=torch.float32, device="cuda")
+    b = torch.zeros_like(a)
+    dt, fl = sv.step1d_noalloc(P, n, 1.0, a.data_ptr(), b.data_ptr())
+    assert dt == 0.0 and fl & sv.FLAG_NONPHYS
+    assert not b.any()
