@@ -215,7 +215,7 @@ __device__ __forceinline__ void cfl(const P<float>& k, const f2 (&N)[4], int mas
   const float vx = fabsf(q.v.x), vy = fabsf(q.v.y);
   if (mask & 1) {
     if ((N[0].x > 0.0f) && (q.p.x > 0.0f)) {
-      smax = fmaxf(smax, fmaxf(2.0f * vx, vx + c.x));
+      smax = fmaxf(smax, fmaxf(2.0f * vx, __fadd_rn(vx, c.x)));
       if (SRC != 0) akey = fmaxf(akey, key.x);
     } else {
       flags |= FLAG_NONPHYS;
@@ -223,7 +223,7 @@ __device__ __forceinline__ void cfl(const P<float>& k, const f2 (&N)[4], int mas
   }
   if (mask & 2) {
     if ((N[0].y > 0.0f) && (q.p.y > 0.0f)) {
-      smax = fmaxf(smax, fmaxf(2.0f * vy, vy + c.y));
+      smax = fmaxf(smax, fmaxf(2.0f * vy, __fadd_rn(vy, c.y)));
       if (SRC != 0) akey = fmaxf(akey, key.y);
     } else {
       flags |= FLAG_NONPHYS;

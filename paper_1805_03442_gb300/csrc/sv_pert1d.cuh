@@ -85,7 +85,7 @@ __device__ __forceinline__ void bound(const P<float>& k, const float (&u)[4], fl
   }
   const float vmag = fabsf(q.v);
   const float c = Ar<float>::sqrt_pos(k.gamma * q.p * q.ir);
-  smax = fmaxf(smax, fmaxf(2.0f * vmag, vmag + c));
+  smax = fmaxf(smax, fmaxf(2.0f * vmag, __fadd_rn(vmag, c)));
   if (SRC != 0) akey = fmaxf(akey, tau_key(k, q.rho, q.p * q.ir));
 }
 
@@ -259,7 +259,7 @@ __device__ __forceinline__ void cfl(const P<float>& k, const f2 (&N)[4], int mas
   const float vx = fabsf(q.v.x), vy = fabsf(q.v.y);
   if (mask & 1) {
     if ((q.rho.x > 0.0f) && (q.p.x > 0.0f)) {
-      smax = fmaxf(smax, fmaxf(2.0f * vx, vx + c.x));
+      smax = fmaxf(smax, fmaxf(2.0f * vx, __fadd_rn(vx, c.x)));
       if (SRC != 0) akey = fmaxf(akey, key.x);
     } else {
       flags |= FLAG_NONPHYS;
@@ -267,7 +267,7 @@ __device__ __forceinline__ void cfl(const P<float>& k, const f2 (&N)[4], int mas
   }
   if (mask & 2) {
     if ((q.rho.y > 0.0f) && (q.p.y > 0.0f)) {
-      smax = fmaxf(smax, fmaxf(2.0f * vy, vy + c.y));
+      smax = fmaxf(smax, fmaxf(2.0f * vy, __fadd_rn(vy, c.y)));
       if (SRC != 0) akey = fmaxf(akey, key.y);
     } else {
       flags |= FLAG_NONPHYS;

@@ -81,7 +81,7 @@ __device__ __forceinline__ void bound(const P<float>& k, const float (&u)[DIM + 
   }
   const float vmag = speed_of(q.v2);
   const float c = Ar<float>::sqrt_pos(k.gamma * q.p * q.ir);
-  smax = fmaxf(smax, fmaxf(2.0f * vmag, vmag + c));
+  smax = fmaxf(smax, fmaxf(2.0f * vmag, __fadd_rn(vmag, c)));
   if (SRC != 0) akey = fmaxf(akey, tau_key(k, q.rho, q.p * q.ir));
 }
 
@@ -119,19 +119,19 @@ __device__ __forceinline__ Prim<DIM> prim(const P<float>& k, const f2 (&u)[DIM +
   return q;
 }
 
-template <int DIM, int A>
-__device__ __forceinline__ void flux(const P<float>& k, const f2 (&u)[DIM + 3], const Prim<DIM>& q,
-                                     f2 (&F)[DIM + 3]) {
-  F[0] = u[1 + A];
-#pragma unroll
-  for (int b = 0; b < DIM; ++b) F[1 + b] = b == A ? fma(u[1 + b], q.v[A], q.dp) : mul(u[1 + b], q.v[A]);
-  F[1 + DIM] = mul(q.v[A], add(splat(k.h0), add(u[1 + DIM], q.dp)));
-  F[2 + DIM] = mul(q.v[A], add(splat(k.ev0), u[2 + DIM]));
+// what v carries of the energies: those of U_ref added to the state's
+template <int DIM>
+__device__ __forceinline__ f2 carried_E(const P<float>& k, const f2 (&u)[DIM + 3], const Prim<DIM>& q) {
+  return add(splat(k.h0), add(u[1 + DIM], q.dp));
+}
+template <int DIM>
+__device__ __forceinline__ f2 carried_Ev(const P<float>& k, const f2 (&u)[DIM + 3]) {
+  return add(splat(k.ev0), u[2 + DIM]);
 }
 
-template <int DIM, int A>
+template <int DIM, int A, bool FIRST>
 __device__ __forceinline__ void dflux(const P<float>& k, const f2 (&u)[DIM + 3],
-                                      const f2 (&d)[DIM + 3], f2 (&dF)[DIM + 3], bool& ok0,
+                                      const f2 (&d)[DIM + 3], f2 (&div)[DIM + 3], bool& ok0,
                                       bool& ok1) {
   constexpr int NF = DIM + 3;
   f2 a[NF], b[NF];
@@ -141,11 +141,9 @@ __device__ __forceinline__ void dflux(const P<float>& k, const f2 (&u)[DIM + 3],
     b[f] = fma(splat(-0.5f), d[f], u[f]);
   }
   const Prim<DIM> pa = prim<DIM>(k, a), pb = prim<DIM>(k, b);
-  f2 Fa[NF], Fb[NF];
-  flux<DIM, A>(k, a, pa, Fa);
-  flux<DIM, A>(k, b, pb, Fb);
-#pragma unroll
-  for (int f = 0; f < NF; ++f) dF[f] = sub(Fa[f], Fb[f]);
+  pkn::add_dflux<DIM, A, FIRST>(d, a, b, pa.v[A], pb.v[A], sub(pa.dp, pb.dp), carried_E<DIM>(k, a, pa),
+                                carried_Ev<DIM>(k, a), carried_E<DIM>(k, b, pb),
+                                carried_Ev<DIM>(k, b), div);
   ok0 = ok0 && fminf(fminf(pa.rho.x, pa.p.x), fminf(pb.rho.x, pb.p.x)) > 0.0f;
   ok1 = ok1 && fminf(fminf(pa.rho.y, pa.p.y), fminf(pb.rho.y, pb.p.y)) > 0.0f;
 }
@@ -193,13 +191,10 @@ __device__ __forceinline__ void hll(const P<float>& k, f2 (&L)[DIM + 3], f2 (&R)
   const f2 qL = add(pl.v[A], cL), qR = add(pr.v[A], cR);
   const f2 nsl = pair(fmaxf(fmaxf(mL.x, mR.x), 0.0f), fmaxf(fmaxf(mL.y, mR.y), 0.0f));
   const f2 sr = pair(fmaxf(fmaxf(qL.x, qR.x), 0.0f), fmaxf(fmaxf(qL.y, qR.y), 0.0f));
-  f2 FL[NF], FR[NF];
-  flux<DIM, A>(k, L, pl, FL);
-  flux<DIM, A>(k, R, pr, FR);
   const f2 inv = rcp(add(sr, nsl));
   const f2 wl = mul(sr, inv), wr = mul(nsl, inv), wd = mul(mul(nsl, sr), inv);
-#pragma unroll
-  for (int f = 0; f < NF; ++f) F[f] = fma(wd, sub(L[f], R[f]), fma(wl, FL[f], mul(wr, FR[f])));
+  pkn::hll_sum<DIM, A>(L, R, wl, wr, wd, pl.v[A], pr.v[A], pl.dp, pr.dp, carried_E<DIM>(k, L, pl),
+                       carried_Ev<DIM>(k, L), carried_E<DIM>(k, R, pr), carried_Ev<DIM>(k, R), F);
 }
 
 template <int DIM, int SRC>
@@ -216,7 +211,7 @@ __device__ __forceinline__ void cfl(const P<float>& k, const f2 (&N)[DIM + 3], i
   const float vx = speed_of(v2.x), vy = speed_of(v2.y);
   if (mask & 1) {
     if ((q.rho.x > 0.0f) && (q.p.x > 0.0f)) {
-      smax = fmaxf(smax, fmaxf(2.0f * vx, vx + c.x));
+      smax = fmaxf(smax, fmaxf(2.0f * vx, __fadd_rn(vx, c.x)));
       if (SRC != 0) akey = fmaxf(akey, key.x);
     } else {
       flags |= FLAG_NONPHYS;
@@ -224,7 +219,7 @@ __device__ __forceinline__ void cfl(const P<float>& k, const f2 (&N)[DIM + 3], i
   }
   if (mask & 2) {
     if ((q.rho.y > 0.0f) && (q.p.y > 0.0f)) {
-      smax = fmaxf(smax, fmaxf(2.0f * vy, vy + c.y));
+      smax = fmaxf(smax, fmaxf(2.0f * vy, __fadd_rn(vy, c.y)));
       if (SRC != 0) akey = fmaxf(akey, key.y);
     } else {
       flags |= FLAG_NONPHYS;
@@ -241,12 +236,12 @@ namespace sv {
 // full-state pair arithmetic (sv_pairnd.cuh), PP 3 the perturbation layout.
 namespace pknx {
 
-template <int DIM, int PP, int A>
+template <int DIM, int PP, int A, bool FIRST>
 __device__ __forceinline__ void dflux(const P<float>& k, const pk::f2 (&u)[DIM + 3],
-                                      const pk::f2 (&d)[DIM + 3], pk::f2 (&dF)[DIM + 3], bool& ok0,
+                                      const pk::f2 (&d)[DIM + 3], pk::f2 (&div)[DIM + 3], bool& ok0,
                                       bool& ok1) {
-  if constexpr (PP == 3) pknps::dflux<DIM, A>(k, u, d, dF, ok0, ok1);
-  else pkn::dflux<DIM, PP, A>(k, u, d, dF, ok0, ok1);
+  if constexpr (PP == 3) pknps::dflux<DIM, A, FIRST>(k, u, d, div, ok0, ok1);
+  else pkn::dflux<DIM, PP, A, FIRST>(k, u, d, div, ok0, ok1);
 }
 
 template <int DIM, int PP, int SRC>

@@ -45,6 +45,9 @@ __device__ __forceinline__ float speed_of(float v2) {
 // Signal speed, tau key and physicality of one updated float state
 // (dim-generic), folded into per-thread maxima.
 // `kin2` = rho |v|^2, `vmag` = |v|.  SRC 0 (frozen) has no tau bound.
+// The sum |v| + c is rounded by itself here and in every other bound: left to
+// the compiler, c = x rsqrt(x) fuses into it in some kernels and not in others,
+// and a state's dt then depends on which kernel bounded it.
 template <int PP, int SRC>
 __device__ __forceinline__ void cfl_cell(const P<float>& k, float rho, float kin2, float vmag,
                                          float E, float Ev, float& smax, float& akey,
@@ -56,7 +59,7 @@ __device__ __forceinline__ void cfl_cell(const P<float>& k, float rho, float kin
     return;
   }
   const float c = Ar<float>::sqrt_pos(k.gamma * p * ir);
-  smax = fmaxf(smax, fmaxf(2.0f * vmag, vmag + c));
+  smax = fmaxf(smax, fmaxf(2.0f * vmag, __fadd_rn(vmag, c)));
   if (SRC != 0) akey = fmaxf(akey, tau_key(k, rho, p * ir));
 }
 

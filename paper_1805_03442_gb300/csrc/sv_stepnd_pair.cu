@@ -140,22 +140,30 @@ stepnd_pair_kernel(const KParams kp, float* __restrict__ bufA, float* __restrict
   // plane p lives in component (p - q0) & 1 of ring pair (p - q0 + 4) / 2
   // mod D/2.  Copy plane p of the own column (p <= q1 + 3) and of the second
   // ring (p <= q1 + 2) into its place; always commit a group.
+  // Cell c of field f, as the field's uniform base and an unsigned 32-bit byte
+  // offset that the fields share (a field's bytes are below 2^32).  Signed cell
+  // offsets with f ncell added to them took 64-bit address arithmetic per access:
+  // 8192^2 1227 -> 1216 us per step.
+  auto at = [&](auto* U, int f, I c) {
+    auto* const field = U + f * ncell;
+    return reinterpret_cast<decltype(field)>((char*)field + 4u * (uint32_t)c);
+  };
   auto issue = [&](I p) {
     const int r = (int)(p - q0 + 4), ps = (r >> 1) & (DP - 1), h = r & 1;
     if (p <= q1 + 3) {
       bool fy;
       const I o = plane_of(p, fy) * plane;
 #pragma unroll
-      for (int f = 0; f < NF; ++f) cp_async<4>(half_of(&sR[ps][f][tid], h), Uin + f * ncell + o + col);
+      for (int f = 0; f < NF; ++f) cp_async<4>(half_of(&sR[ps][f][tid], h), at(Uin, f, o + col));
       if (p <= q1 + 2) {
         if (ringx)
 #pragma unroll
           for (int f = 0; f < NF; ++f)
-            cp_async<4>(half_of(&sH[ps][f][hx], h), Uin + f * ncell + o + col_rx);
+            cp_async<4>(half_of(&sH[ps][f][hx], h), at(Uin, f, o + col_rx));
         if (ringy)
 #pragma unroll
           for (int f = 0; f < NF; ++f)
-            cp_async<4>(half_of(&sH[ps][f][hy], h), Uin + f * ncell + o + col_ry);
+            cp_async<4>(half_of(&sH[ps][f][hy], h), at(Uin, f, o + col_ry));
       }
     }
     cp_async_commit();
@@ -244,17 +252,11 @@ stepnd_pair_kernel(const KParams kp, float* __restrict__ bufA, float* __restrict
         d[AM][f] = pk::pair(pk::slope<LIM>(A.x, B.x), pk::slope<LIM>(A.y, B.y));
       }
     }
-    f2 div[NF], dF[NF];
+    f2 div[NF];
     bool ok0 = true, ok1 = true;
-    pknx::dflux<DIM, PP, 0>(k, X, d[0], div, ok0, ok1);
-    pknx::dflux<DIM, PP, 1>(k, X, d[1], dF, ok0, ok1);
-#pragma unroll
-    for (int f = 0; f < NF; ++f) div[f] = pk::add(div[f], dF[f]);
-    if (DIM == 3) {
-      pknx::dflux<DIM, PP, DIM == 3 ? 2 : 1>(k, X, d[AM], dF, ok0, ok1);
-#pragma unroll
-      for (int f = 0; f < NF; ++f) div[f] = pk::add(div[f], dF[f]);
-    }
+    pknx::dflux<DIM, PP, 0, true>(k, X, d[0], div, ok0, ok1);
+    pknx::dflux<DIM, PP, 1, false>(k, X, d[1], div, ok0, ok1);
+    if (DIM == 3) pknx::dflux<DIM, PP, DIM == 3 ? 2 : 1, false>(k, X, d[AM], div, ok0, ok1);
     if (!(ok0 && ok1)) {
 #pragma unroll
       for (int f = 0; f < NF; ++f) {
@@ -400,8 +402,8 @@ stepnd_pair_kernel(const KParams kp, float* __restrict__ bufA, float* __restrict
       const I oa = plane_of(q - 2, fy) * plane + col, ob = plane_of(q - 1, fy) * plane + col;
 #pragma unroll
       for (int f = 0; f < NF; ++f) {
-        Uout[f * ncell + oa] = Nw[f].x;
-        if (two) Uout[f * ncell + ob] = Nw[f].y;
+        *at(Uout, f, oa) = Nw[f].x;
+        if (two) *at(Uout, f, ob) = Nw[f].y;
       }
       pknx::cfl<DIM, PP, SRC>(k, Nw, two ? 3 : 1, smax, akey, flags);
     }
@@ -419,8 +421,14 @@ stepnd_pair_kernel(const KParams kp, float* __restrict__ bufA, float* __restrict
   reduce_and_finalize<float, NT>(ctl, kp, smax, akey, flags, true);
 }
 
-// Tiles of the pair kernel: 128 threads along x (126 interior cells), 166-168
-// registers, 3 blocks per SM (a budget of 4 spills).
+// Tiles of the pair kernel: 128 threads along x (126 interior cells), 162-168
+// registers, 3 blocks per SM (a budget of 4 spills).  It is bound by the issue
+// slots and the FMA pipe its packed operations hold for two cycles each
+// (profiles/stepnd2d_fp32_4096x4096.md): folding the fluxes into the sums that use
+// them and the 32-bit offsets took 8192^2 from 1227 to 1185 us per step (FP32;
+// 2000 x 1500 in compensated float 80.6 -> 77.0).  192 threads x 2 blocks 1259 us,
+// 96 x 4 1224 (1000 x 1000 with walls 45.9 -> 63.8); the transverse fluxes left in
+// shared memory for the next iteration, two barriers instead of three, 1251 us.
 template <int DIM> struct PairCfg;
 template <> struct PairCfg<2> { static constexpr int TX = 128, TY = 1, MINB = 3, SEG = 256; };
 
