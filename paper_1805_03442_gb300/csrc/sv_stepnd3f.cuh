@@ -318,7 +318,11 @@ stepnd3f_kernel(const KParams kp, float* __restrict__ bufA, float* __restrict__ 
     }
     __syncthreads();
     f2 Fx[NP], Fy[NP];
-    {
+    // Compensated pressure: none on the two planes around the segment, whose fluxes
+    // nothing reads (201 x 150 x 170, 19 planes per segment: 321 -> 307.5 us per
+    // step).  The branch costs the others more than it saves (float 512^3 5479 ->
+    // 5544, 256^3 792 -> 794, perturbations 157.9 -> 158.2).
+    if (PP != 2 || (q >= q0 && q < q1)) {
       f2 l[NP], r[NP];
 #pragma unroll
       for (int p = 0; p < NP; ++p) {
@@ -348,13 +352,13 @@ stepnd3f_kernel(const KParams kp, float* __restrict__ bufA, float* __restrict__ 
                     }
                   },
                   Fy);
+#pragma unroll
+      for (int p = 0; p < NP; ++p) {
+        sF[0][p][tid] = Fx[p];
+        sF[1][p][tid] = Fy[p];
+      }
     }
     // d. transverse flux divergence of plane q
-#pragma unroll
-    for (int p = 0; p < NP; ++p) {
-      sF[0][p][tid] = Fx[p];
-      sF[1][p][tid] = Fy[p];
-    }
     __syncthreads();
     f2 Dq[NP];
 #pragma unroll
