@@ -331,10 +331,8 @@ int write_state_host(sv_solver* s, const H* host_soa, double t) {
     src = (const H*)s->staging;
   }
   SV_TRY(ctl_reset_launch(s->ctl, t, s->stream));
-  SV_TRY(to_state_launch(s->p.precision, src, s->buf[0], s->buf[1], s->ctl, (int64_t)count,
-                         s->stream, s->kp.ref, s->nf));
-  SV_TRY(dt_reduce_launch(s->p.precision, s->dim, s->kp, s->buf[0], s->buf[1], s->ctl, s->ncell,
-                          s->stream));
+  SV_TRY(upload_launch(s->p.precision, s->dim, s->kp, src, s->buf[0], s->buf[1], s->ctl, s->ncell,
+                       s->stream));
   return SV_OK;
 }
 

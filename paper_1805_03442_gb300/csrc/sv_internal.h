@@ -109,17 +109,17 @@ cudaError_t dt_reduce_launch(int precision, int dim, const KParams& kp, const vo
                              const void* b, Ctl* ctl, int64_t ncell, cudaStream_t st);
 cudaError_t set_target_launch(int precision, Ctl* ctl, double t_end, const KParams& kp,
                               cudaStream_t st);
-// Host-format (double, full state) <-> device state; `ref` (4 values) is the
-// reference state the perturbation layout PREC_FP32_PS subtracts, unused otherwise.
-cudaError_t to_state_launch(int precision, const double* src, void* a, void* b, Ctl* ctl,
-                            int64_t count, cudaStream_t st, const double* ref = nullptr,
-                            int nf = 4);
+// Upload of a host-format (double or float) full state: conversion, and the dt of
+// the state it leaves in the same pass (kp.ref: the reference state that the
+// perturbation layout PREC_FP32_PS subtracts).
+cudaError_t upload_launch(int precision, int dim, const KParams& kp, const double* src, void* a,
+                          void* b, Ctl* ctl, int64_t ncell, cudaStream_t st);
+cudaError_t upload_launch(int precision, int dim, const KParams& kp, const float* src, void* a,
+                          void* b, Ctl* ctl, int64_t ncell, cudaStream_t st);
+// Device state -> host format; `ref` as kp.ref above.
 cudaError_t from_state_launch(int precision, const void* a, const void* b, const Ctl* ctl,
-                              double* dst, int64_t count, cudaStream_t st,
-                              const double* ref = nullptr, int nf = 4);
-// The same with float host-format buffers (sv_write_state_f32 / sv_read_state_f32).
-cudaError_t to_state_launch(int precision, const float* src, void* a, void* b, Ctl* ctl,
-                            int64_t count, cudaStream_t st, const double* ref, int nf);
+                              double* dst, int64_t count, cudaStream_t st, const double* ref,
+                              int nf);
 cudaError_t from_state_launch(int precision, const void* a, const void* b, const Ctl* ctl,
                               float* dst, int64_t count, cudaStream_t st, const double* ref,
                               int nf);

@@ -56,11 +56,33 @@ cudaError_t set_target_launch(int precision, Ctl* ctl, double t_end, const KPara
   return cudaGetLastError();
 }
 
+// Eq. 16 bound of one state, folded into acc.
+template <typename R, int PP, int DIM>
+__device__ __forceinline__ void fold_bound(const P<R>& k, const R (&u)[DIM + 3], Acc<R>& acc) {
+  if constexpr (PP == 3 || std::is_same<R, double>::value) {
+    // the perturbation layout, and double
+    if constexpr (DIM == 1) cell_bound<PP, 1>(k, u, acc);
+    else if constexpr (PP == 3) psn::bound<DIM, 1>(k, u, acc.smax, acc.akey, acc.flags);
+    else d64::bound<DIM, 1>(k, u, acc);
+  } else {
+    const R ir = Ar<R>::rcp(u[0]);
+    R kin2 = 0, v2 = 0;
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) {
+      const R v = u[1 + d] * ir;
+      kin2 = fmaf(u[1 + d], v, kin2);
+      v2 = fmaf(v, v, v2);
+    }
+    const R vmag = DIM == 1 ? fabsf(u[1] * ir) : speed_of(v2);
+    cfl_cell<PP, 1>(k, u[0], kin2, vmag, u[1 + DIM], u[2 + DIM], acc.smax, acc.akey, acc.flags);
+  }
+}
+
 // dt of the current state (no step): same per-cell bound and finalize as the
 // step kernels.
-template <typename R, int PP>
+template <typename R, int PP, int DIM>
 __global__ void __launch_bounds__(NTU) dt_reduce_kernel(const KParams kp, const R* a, const R* b,
-                                                        Ctl* ctl, int dim, int64_t ncell) {
+                                                        Ctl* ctl, int64_t ncell) {
   __shared__ float s_word;
   if (threadIdx.x == 0) s_word = 0.0f;
   __syncthreads();
@@ -69,35 +91,10 @@ __global__ void __launch_bounds__(NTU) dt_reduce_kernel(const KParams kp, const 
   Acc<R> acc(&s_word);
   for (int64_t i = (int64_t)blockIdx.x * NTU + threadIdx.x; i < ncell;
        i += (int64_t)gridDim.x * NTU) {
-    if constexpr (PP == 3 || std::is_same<R, double>::value) {
-      // the perturbation layout, and double
-      if (dim == 1) {
-        const R u[4] = {U[i], U[ncell + i], U[2 * ncell + i], U[3 * ncell + i]};
-        cell_bound<PP, 1>(k, u, acc);
-      } else if (dim == 2) {
-        R u[5];
-        for (int f = 0; f < 5; ++f) u[f] = U[f * ncell + i];
-        if constexpr (PP == 3) psn::bound<2, 1>(k, u, acc.smax, acc.akey, acc.flags);
-        else d64::bound<2, 1>(k, u, acc);
-      } else {
-        R u[6];
-        for (int f = 0; f < 6; ++f) u[f] = U[f * ncell + i];
-        if constexpr (PP == 3) psn::bound<3, 1>(k, u, acc.smax, acc.akey, acc.flags);
-        else d64::bound<3, 1>(k, u, acc);
-      }
-    } else {
-      const R rho = U[i];
-      const R ir = Ar<R>::rcp(rho);
-      R kin2 = 0, v2 = 0;
-      for (int d = 0; d < dim; ++d) {
-        const R m = U[(1 + d) * ncell + i], v = m * ir;
-        kin2 += m * v;
-        v2 += v * v;
-      }
-      const R vmag = dim == 1 ? fabsf(U[ncell + i] * ir) : speed_of(v2);
-      cfl_cell<PP, 1>(k, rho, kin2, vmag, U[(1 + dim) * ncell + i], U[(2 + dim) * ncell + i],
-                      acc.smax, acc.akey, acc.flags);
-    }
+    R u[DIM + 3];
+#pragma unroll
+    for (int f = 0; f < DIM + 3; ++f) u[f] = U[f * ncell + i];
+    fold_bound<R, PP, DIM>(k, u, acc);
   }
   reduce_and_finalize<R, NTU>(ctl, kp, acc.smax, acc.akey, acc.flags, false);
 }
@@ -111,82 +108,30 @@ static int grid_small(int64_t count) {
   return g < 1 ? 1 : (int)g;
 }
 
+template <typename R, int PP>
+void dt_reduce_dim(int dim, const KParams& kp, const void* a, const void* b, Ctl* ctl,
+                   int64_t ncell, cudaStream_t st) {
+  const int g = grid_small(ncell);
+  const R *x = (const R*)a, *y = (const R*)b;
+  if (dim == 1) dt_reduce_kernel<R, PP, 1><<<g, NTU, 0, st>>>(kp, x, y, ctl, ncell);
+  else if (dim == 2) dt_reduce_kernel<R, PP, 2><<<g, NTU, 0, st>>>(kp, x, y, ctl, ncell);
+  else dt_reduce_kernel<R, PP, 3><<<g, NTU, 0, st>>>(kp, x, y, ctl, ncell);
+}
+
 cudaError_t dt_reduce_launch(int precision, int dim, const KParams& kp, const void* a,
                              const void* b, Ctl* ctl, int64_t ncell, cudaStream_t st) {
-  const int g = grid_small(ncell);
   switch (precision) {
-    case PREC_FP64:
-      dt_reduce_kernel<double, 0><<<g, NTU, 0, st>>>(kp, (const double*)a, (const double*)b, ctl,
-                                                     dim, ncell);
-      break;
+    case PREC_FP64: dt_reduce_dim<double, 0>(dim, kp, a, b, ctl, ncell, st); break;
     case PREC_FP32_P64:
-    case PREC_FP32_PC:
-      dt_reduce_kernel<float, 2><<<g, NTU, 0, st>>>(kp, (const float*)a, (const float*)b, ctl,
-                                                    dim, ncell);
-      break;
-    case PREC_FP32_PS:
-      dt_reduce_kernel<float, 3><<<g, NTU, 0, st>>>(kp, (const float*)a, (const float*)b, ctl,
-                                                    dim, ncell);
-      break;
-    default:
-      dt_reduce_kernel<float, 0><<<g, NTU, 0, st>>>(kp, (const float*)a, (const float*)b, ctl,
-                                                    dim, ncell);
+    case PREC_FP32_PC: dt_reduce_dim<float, 2>(dim, kp, a, b, ctl, ncell, st); break;
+    case PREC_FP32_PS: dt_reduce_dim<float, 3>(dim, kp, a, b, ctl, ncell, st); break;
+    default: dt_reduce_dim<float, 0>(dim, kp, a, b, ctl, ncell, st);
   }
   return cudaGetLastError();
 }
 
-// Host-format (double) <-> state conversion.  `src` / `dst` is a device
-// staging buffer or the device view of mapped pinned host memory (then the
-// kernel itself moves the bytes over the host link).  Pairs of elements go as
-// one 16-byte double2 access where both sides are aligned for it.
-template <typename R> struct Vec2;
-template <> struct Vec2<float> { using T = float2; };
-template <> struct Vec2<double> { using T = double2; };
-
-template <typename H, typename R>
-__global__ void to_state_kernel(const H* src, R* a, R* b, const Ctl* ctl, int64_t count) {
-  R* U = vload(&ctl->cur) ? b : a;
-  using R2 = typename Vec2<R>::T;
-  using H2 = typename Vec2<H>::T;
-  const int64_t i0 = (int64_t)blockIdx.x * NTU + threadIdx.x, di = (int64_t)gridDim.x * NTU;
-  if (((uintptr_t)src & (sizeof(H2) - 1)) == 0 && ((uintptr_t)U & (sizeof(R2) - 1)) == 0) {
-    const int64_t n2 = count / 2;
-    for (int64_t i = i0; i < n2; i += di) {
-      const H2 v = reinterpret_cast<const H2*>(src)[i];
-      R2 w;
-      w.x = (R)v.x;
-      w.y = (R)v.y;
-      reinterpret_cast<R2*>(U)[i] = w;
-    }
-    if (i0 == 0 && (count & 1)) U[count - 1] = (R)src[count - 1];
-  } else {
-    for (int64_t i = i0; i < count; i += di) U[i] = (R)src[i];
-  }
-}
-
-template <typename H, typename R>
-__global__ void from_state_kernel(const R* a, const R* b, const Ctl* ctl, H* dst, int64_t count) {
-  const R* U = vload(&ctl->cur) ? b : a;
-  using R2 = typename Vec2<R>::T;
-  using H2 = typename Vec2<H>::T;
-  const int64_t i0 = (int64_t)blockIdx.x * NTU + threadIdx.x, di = (int64_t)gridDim.x * NTU;
-  if (((uintptr_t)dst & (sizeof(H2) - 1)) == 0 && ((uintptr_t)U & (sizeof(R2) - 1)) == 0) {
-    const int64_t n2 = count / 2;
-    for (int64_t i = i0; i < n2; i += di) {
-      const R2 w = reinterpret_cast<const R2*>(U)[i];
-      H2 v;
-      v.x = (H)w.x;
-      v.y = (H)w.y;
-      reinterpret_cast<H2*>(dst)[i] = v;
-    }
-    if (i0 == 0 && (count & 1)) dst[count - 1] = (H)U[count - 1];
-  } else {
-    for (int64_t i = i0; i < count; i += di) dst[i] = (H)U[i];
-  }
-}
-
-// The perturbation layout (SV_FP32_PS): element i of field f = i / ncell holds
-// (float)(U - ref[f]) (the difference taken in double); nf = 4, 5 or 6 fields.
+// The perturbation layout (SV_FP32_PS) holds (float)(U - ref[f]) of field f, the
+// difference taken in double; nf = 4, 5 or 6 fields.
 struct RefN {
   double v[6];
 };
@@ -198,22 +143,139 @@ RefN ref_of(const double* ref, int nf) {
   return r;
 }
 
-template <typename H>
-__global__ void to_state_ps_kernel(const H* src, float* a, float* b, const Ctl* ctl,
-                                   int64_t count, int64_t ncell, RefN ref) {
-  float* U = vload(&ctl->cur) ? b : a;
-  for (int64_t i = (int64_t)blockIdx.x * NTU + threadIdx.x; i < count;
-       i += (int64_t)gridDim.x * NTU)
-    U[i] = (float)((double)src[i] - ref.v[i / ncell]);
+// V consecutive elements in accesses of at most 16 bytes.
+template <int V, typename T>
+__device__ __forceinline__ void load_v(const T* p, T (&v)[V]) {
+  if constexpr (std::is_same<T, float>::value && V == 4) {
+    const float4 q = *reinterpret_cast<const float4*>(p);
+    v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+  } else if constexpr (std::is_same<T, float>::value) {
+    const float2 q = *reinterpret_cast<const float2*>(p);
+    v[0] = q.x; v[1] = q.y;
+  } else {
+#pragma unroll
+    for (int i = 0; i < V; i += 2) {
+      const double2 q = *reinterpret_cast<const double2*>(p + i);
+      v[i] = q.x; v[i + 1] = q.y;
+    }
+  }
+}
+template <int V, typename T>
+__device__ __forceinline__ void store_v(T* p, const T (&v)[V]) {
+  if constexpr (std::is_same<T, float>::value && V == 4) {
+    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+  } else if constexpr (std::is_same<T, float>::value) {
+    *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < V; i += 2)
+      *reinterpret_cast<double2*>(p + i) = make_double2(v[i], v[i + 1]);
+  }
+}
+// Host-format (double or float) -> state conversion of an upload, with the dt of
+// the state it leaves.  `src` is a device staging buffer or the device view of
+// mapped pinned host memory (then the kernel itself moves the bytes over the
+// host link, which bounds it).  A thread takes as many consecutive cells as 16
+// bytes of the host format hold, all fields, and bounds them from registers.
+// A second pass over the state for the bound and 8-byte accesses took, ms,
+// against now and a plain copy: 512^3 float 16.7 / 15.3 / 15.2, 8192^2 7.08 / 6.37 / 6.35.
+// Fields that are not all aligned for that (odd cell counts) keep the two
+// passes (to_state_kernel, dt_reduce_kernel): a cell at a time here, 4-byte
+// accesses over the link, took 376 us at 4194301 cells, the two passes 350.
+template <bool PS, typename R, typename H>
+__device__ __forceinline__ R to_state(H v, double ref) {
+  return PS ? (R)((double)v - ref) : (R)v;
 }
 
-template <typename H>
-__global__ void from_state_ps_kernel(const float* a, const float* b, const Ctl* ctl, H* dst,
-                                     int64_t count, int64_t ncell, RefN ref) {
-  const float* U = vload(&ctl->cur) ? b : a;
-  for (int64_t i = (int64_t)blockIdx.x * NTU + threadIdx.x; i < count;
-       i += (int64_t)gridDim.x * NTU)
-    dst[i] = (H)(ref.v[i / ncell] + (double)U[i]);
+template <typename H, typename R, int PP, int DIM>
+__global__ void __launch_bounds__(NTU)
+upload_kernel(const KParams kp, const H* __restrict__ src, R* __restrict__ a, R* __restrict__ b,
+              Ctl* ctl, int64_t ncell, RefN ref) {
+  constexpr int NF = DIM + 3;
+  __shared__ float s_word;
+  if (threadIdx.x == 0) s_word = 0.0f;
+  __syncthreads();
+  R* __restrict__ U = vload(&ctl->cur) ? b : a;
+  const P<R> k(kp);
+  Acc<R> acc(&s_word);
+  const int64_t i0 = (int64_t)blockIdx.x * NTU + threadIdx.x, di = (int64_t)gridDim.x * NTU;
+  constexpr int V = 16 / sizeof(H);
+  for (int64_t i = V * i0; i < ncell; i += V * di) {
+    H h[NF][V];
+    R u[NF][V];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) load_v<V>(src + f * ncell + i, h[f]);
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+#pragma unroll
+      for (int c = 0; c < V; ++c) u[f][c] = to_state<PP == 3, R>(h[f][c], ref.v[f]);
+      store_v<V>(U + f * ncell + i, u[f]);
+    }
+#pragma unroll
+    for (int c = 0; c < V; ++c) {
+      R v[NF];
+#pragma unroll
+      for (int f = 0; f < NF; ++f) v[f] = u[f][c];
+      fold_bound<R, PP, DIM>(k, v, acc);
+    }
+  }
+  reduce_and_finalize<R, NTU>(ctl, kp, acc.smax, acc.akey, acc.flags, false);
+}
+
+// Elements before the first 128-byte boundary of p (at most n).
+template <typename T>
+__device__ __forceinline__ int64_t head_of(const T* p, int64_t n) {
+  const int64_t h = (int64_t)((128 - ((uintptr_t)p & 127)) & 127) / (int64_t)sizeof(T);
+  return h < n ? h : n;
+}
+
+// Host format -> state without the dt, and state -> host format of a download.  A
+// lane's accesses on the host's side are single ones of 16 bytes from the first
+// line boundary on (two of them 32 bytes apart per lane halved the rate of
+// a double download, 199 -> 410 us for 32 MB; rows begun at a 16-byte boundary
+// inside a line took 306 us instead of 282 at 3000001 cells); those of the state, whose rows
+// need not be aligned to the host's, are elements.  Fields are alike but for the
+// reference state of the perturbation layout (PS), which takes one row of
+// blocks per field; otherwise n counts the elements of all.
+template <typename H, typename R, bool PS>
+__global__ void __launch_bounds__(NTU)
+to_state_kernel(const H* src, R* a, R* b, const Ctl* ctl, int64_t n, RefN ref) {
+  const int f = PS ? blockIdx.y : 0;
+  R* const U = (vload(&ctl->cur) ? b : a) + f * n;
+  const double r = ref.v[f];
+  const H* const in = src + f * n;
+  constexpr int V = 16 / sizeof(H);
+  const int64_t i0 = (int64_t)blockIdx.x * NTU + threadIdx.x, di = (int64_t)gridDim.x * NTU;
+  const int64_t head = head_of(in, n), nv = head + (n - head) / V * V;
+  if (i0 < head) U[i0] = to_state<PS, R>(in[i0], r);
+  for (int64_t i = head + V * i0; i < nv; i += V * di) {
+    H h[V];
+    load_v<V>(in + i, h);
+#pragma unroll
+    for (int c = 0; c < V; ++c) U[i + c] = to_state<PS, R>(h[c], r);
+  }
+  if (nv + i0 < n) U[nv + i0] = to_state<PS, R>(in[nv + i0], r);
+}
+
+template <typename H, typename R, bool PS>
+__global__ void __launch_bounds__(NTU)
+from_state_kernel(const R* a, const R* b, const Ctl* ctl, H* dst, int64_t n, RefN ref) {
+  const int f = PS ? blockIdx.y : 0;
+  const R* const U = (vload(&ctl->cur) ? b : a) + f * n;
+  const double r = ref.v[f];
+  H* const out = dst + f * n;
+  auto host = [&](R v) { return PS ? (H)(r + (double)v) : (H)v; };
+  constexpr int V = 16 / sizeof(H);
+  const int64_t i0 = (int64_t)blockIdx.x * NTU + threadIdx.x, di = (int64_t)gridDim.x * NTU;
+  const int64_t head = head_of(out, n), nv = head + (n - head) / V * V;
+  if (i0 < head) out[i0] = host(U[i0]);
+  for (int64_t i = head + V * i0; i < nv; i += V * di) {
+    H h[V];
+#pragma unroll
+    for (int c = 0; c < V; ++c) h[c] = host(U[i + c]);
+    store_v<V>(out + i, h);
+  }
+  if (nv + i0 < n) out[nv + i0] = host(U[nv + i0]);
 }
 
 // Raw copies of the current state buffer (`words` 4-byte words) to / from
@@ -236,47 +298,62 @@ cudaError_t raw_state_launch(void* a, void* b, const Ctl* ctl, void* other, int6
   return cudaGetLastError();
 }
 
-template <typename H>
-cudaError_t to_state_impl(int precision, const H* src, void* a, void* b, Ctl* ctl, int64_t count,
-                          cudaStream_t st, const double* ref, int nf) {
-  const int g = grid_small(count);
-  if (precision == PREC_FP32_PS) {
-    to_state_ps_kernel<H><<<g, NTU, 0, st>>>(src, (float*)a, (float*)b, ctl, count, count / nf,
-                                             ref_of(ref, nf));
-    return cudaGetLastError();
+template <typename H, typename R, int PP>
+void upload_dim(int dim, const KParams& kp, const H* src, void* a, void* b, Ctl* ctl, int64_t ncell,
+                cudaStream_t st) {
+  const int nf = dim + 3;
+  const RefN ref = ref_of(kp.ref, nf);
+  R *x = (R*)a, *y = (R*)b;
+  if (((uintptr_t)src | (uintptr_t)a | (uintptr_t)b) % 16 != 0 || ncell % (16 / sizeof(H)) != 0) {
+    const int64_t n = PP == 3 ? ncell : nf * ncell;
+    const dim3 g(grid_small((n + 3) / 4), PP == 3 ? nf : 1);
+    to_state_kernel<H, R, PP == 3><<<g, NTU, 0, st>>>(src, x, y, ctl, n, ref);
+    dt_reduce_dim<R, PP>(dim, kp, a, b, ctl, ncell, st);
+    return;
   }
-  if (precision == PREC_FP64)
-    to_state_kernel<H, double><<<g, NTU, 0, st>>>(src, (double*)a, (double*)b, ctl, count);
-  else
-    to_state_kernel<H, float><<<g, NTU, 0, st>>>(src, (float*)a, (float*)b, ctl, count);
+  const int g = grid_small((ncell + 3) / 4);
+  if (dim == 1) upload_kernel<H, R, PP, 1><<<g, NTU, 0, st>>>(kp, src, x, y, ctl, ncell, ref);
+  else if (dim == 2) upload_kernel<H, R, PP, 2><<<g, NTU, 0, st>>>(kp, src, x, y, ctl, ncell, ref);
+  else upload_kernel<H, R, PP, 3><<<g, NTU, 0, st>>>(kp, src, x, y, ctl, ncell, ref);
+}
+
+template <typename H>
+cudaError_t upload_impl(int precision, int dim, const KParams& kp, const H* src, void* a, void* b,
+                        Ctl* ctl, int64_t ncell, cudaStream_t st) {
+  switch (precision) {
+    case PREC_FP64: upload_dim<H, double, 0>(dim, kp, src, a, b, ctl, ncell, st); break;
+    case PREC_FP32_P64:
+    case PREC_FP32_PC: upload_dim<H, float, 2>(dim, kp, src, a, b, ctl, ncell, st); break;
+    case PREC_FP32_PS: upload_dim<H, float, 3>(dim, kp, src, a, b, ctl, ncell, st); break;
+    default: upload_dim<H, float, 0>(dim, kp, src, a, b, ctl, ncell, st);
+  }
   return cudaGetLastError();
 }
 
 template <typename H>
 cudaError_t from_state_impl(int precision, const void* a, const void* b, const Ctl* ctl, H* dst,
                             int64_t count, cudaStream_t st, const double* ref, int nf) {
-  const int g = grid_small(count);
-  if (precision == PREC_FP32_PS) {
-    from_state_ps_kernel<H><<<g, NTU, 0, st>>>((const float*)a, (const float*)b, ctl, dst, count,
-                                               count / nf, ref_of(ref, nf));
-    return cudaGetLastError();
-  }
-  if (precision == PREC_FP64)
-    from_state_kernel<H, double><<<g, NTU, 0, st>>>((const double*)a, (const double*)b, ctl, dst,
-                                                    count);
+  const RefN r = ref_of(ref, nf);
+  const int64_t ncell = count / nf;
+  if (precision == PREC_FP32_PS)
+    from_state_kernel<H, float, true><<<dim3(grid_small((ncell + 3) / 4), nf), NTU, 0, st>>>(
+        (const float*)a, (const float*)b, ctl, dst, ncell, r);
+  else if (precision == PREC_FP64)
+    from_state_kernel<H, double, false><<<grid_small((count + 3) / 4), NTU, 0, st>>>(
+        (const double*)a, (const double*)b, ctl, dst, count, r);
   else
-    from_state_kernel<H, float><<<g, NTU, 0, st>>>((const float*)a, (const float*)b, ctl, dst,
-                                                   count);
+    from_state_kernel<H, float, false><<<grid_small((count + 3) / 4), NTU, 0, st>>>(
+        (const float*)a, (const float*)b, ctl, dst, count, r);
   return cudaGetLastError();
 }
 
-cudaError_t to_state_launch(int precision, const double* src, void* a, void* b, Ctl* ctl,
-                            int64_t count, cudaStream_t st, const double* ref, int nf) {
-  return to_state_impl<double>(precision, src, a, b, ctl, count, st, ref, nf);
+cudaError_t upload_launch(int precision, int dim, const KParams& kp, const double* src, void* a,
+                          void* b, Ctl* ctl, int64_t ncell, cudaStream_t st) {
+  return upload_impl(precision, dim, kp, src, a, b, ctl, ncell, st);
 }
-cudaError_t to_state_launch(int precision, const float* src, void* a, void* b, Ctl* ctl,
-                            int64_t count, cudaStream_t st, const double* ref, int nf) {
-  return to_state_impl<float>(precision, src, a, b, ctl, count, st, ref, nf);
+cudaError_t upload_launch(int precision, int dim, const KParams& kp, const float* src, void* a,
+                          void* b, Ctl* ctl, int64_t ncell, cudaStream_t st) {
+  return upload_impl(precision, dim, kp, src, a, b, ctl, ncell, st);
 }
 cudaError_t from_state_launch(int precision, const void* a, const void* b, const Ctl* ctl,
                               double* dst, int64_t count, cudaStream_t st, const double* ref,
