@@ -31,6 +31,22 @@ namespace sv {
 // Kernels of the two block sizes: 256 threads here, 128 in sv_batch128.cu.
 void* batch_pick256(int limiter, int precision) { return bpick<256>(limiter, precision); }
 
+// The states that the runs are at, to page-locked host memory: blockIdx.x over
+// the runs, blockIdx.y over parts of one.  A run's block of 4 stride elements is
+// a multiple of 128 elements and starts at one.
+static __global__ void __launch_bounds__(256) gather_states_kernel(const RunDev* runs, int nruns,
+                                                            const unsigned char* a,
+                                                            const unsigned char* b,
+                                                            unsigned char* host, int esize) {
+  for (int i = blockIdx.x; i < nruns; i += gridDim.x) {
+    const size_t off = (size_t)runs[i].off * esize;
+    const uint4* const src = (const uint4*)((runs[i].cur ? b : a) + off);
+    uint4* const dst = (uint4*)(host + off);
+    const int n16 = runs[i].stride * 4 * esize / 16;
+    for (int j = blockIdx.y * 256 + threadIdx.x; j < n16; j += gridDim.y * 256) dst[j] = src[j];
+  }
+}
+
 }  // namespace sv
 
 using namespace sv;
@@ -50,12 +66,17 @@ struct sv_batch {
   int* queue = nullptr;
   double* logs = nullptr;
   std::vector<RunDev> host_runs;      // the records as last uploaded
-  // Page-locked copies of what a run leaves: its records and logs, copied behind
-  // the kernel as part of the run, and room for one run's state.  Null (the
-  // reads then copy from the device each time) beyond kMirrorBytes.
+  // Page-locked copies of what a run leaves: its records, logs and states,
+  // copied behind the kernel as part of the run (an upload packs its states there
+  // too).  Null (the reads then copy from the device each time) beyond
+  // kMirrorBytes; `staging` then holds one run's state.  With 256 runs a
+  // copy and a wait per read and a pageable upload took 14 of a sweep's 32 ms
+  // on the host, now 11 of 28.9.
   RunDev* mirror = nullptr;
   double* mirror_logs = nullptr;
   unsigned char* staging = nullptr;
+  void* staging_dev = nullptr;        // its device address
+  bool whole = false;                 // staging holds every run's state
   std::vector<int64_t> n;
   std::vector<int> host_order;        // queue order
   int64_t total_elems = 0;
@@ -143,10 +164,14 @@ void pack_states(const sv_batch* b, const double* host, R* out) {
 }
 
 int upload(sv_batch* b, const double* host) {
-  std::vector<unsigned char> tmp((size_t)b->total_elems * (size_t)b->esize, 0);
-  if (b->esize == 8) pack_states(b, host, (double*)tmp.data());
-  else pack_states(b, host, (float*)tmp.data());
-  SVB_TRY(cudaMemcpyAsync(b->buf[0], tmp.data(), tmp.size(), cudaMemcpyHostToDevice, b->stream));
+  const size_t bytes = (size_t)b->total_elems * (size_t)b->esize;
+  std::vector<unsigned char> tmp;
+  if (b->whole) SVB_TRY(cudaStreamSynchronize(b->stream));   // a run may be copying its states there
+  else tmp.resize(bytes, 0);
+  unsigned char* const packed = b->whole ? b->staging : tmp.data();
+  if (b->esize == 8) pack_states(b, host, (double*)packed);
+  else pack_states(b, host, (float*)packed);
+  SVB_TRY(cudaMemcpyAsync(b->buf[0], packed, bytes, cudaMemcpyHostToDevice, b->stream));
   for (auto& r : b->host_runs) {
     r.t = 0.0;
     r.steps = 0;
@@ -285,6 +310,12 @@ cudaError_t launch_batch(sv_batch* b, cudaStream_t st) {
                   &b->cluster};
   const BatchLaunch l(b->grid / b->cluster, b->cluster, b->nt, st);
   e = cudaLaunchKernelExC(&l.cfg, b->fn, args);
+  if (e == cudaSuccess && b->whole) {
+    gather_states_kernel<<<dim3(nr < 1024 ? nr : 1024, 4), 256, 0, st>>>(
+        b->runs, nr, (const unsigned char*)b->buf[0], (const unsigned char*)b->buf[1],
+        (unsigned char*)b->staging_dev, b->esize);
+    e = cudaGetLastError();
+  }
   if (e == cudaSuccess && b->mirror)
     e = cudaMemcpyAsync(b->mirror, b->runs, sizeof(RunDev) * (size_t)b->nruns,
                         cudaMemcpyDeviceToHost, st);
@@ -434,7 +465,16 @@ int sv_batch_init(const sv_params* p, const sv_run* runs, int64_t nruns,
     };
     lock((void**)&b->mirror, rec);
     if (b->mirror) lock((void**)&b->mirror_logs, log_bytes(b));
-    lock((void**)&b->staging, (size_t)widest);
+    const size_t all = (size_t)b->total_elems * (size_t)b->esize;
+    lock((void**)&b->staging, all);
+    if (b->staging && cudaHostGetDevicePointer(&b->staging_dev, b->staging, 0) != cudaSuccess) {
+      cudaGetLastError();
+      cudaFreeHost(b->staging);
+      b->staging = nullptr;
+    }
+    b->whole = b->staging != nullptr;
+    if (b->whole) memset(b->staging, 0, all);        // the rows' padding
+    else lock((void**)&b->staging, (size_t)widest);
   }
   if (rc == SV_OK) rc = apply_config(b, 0);
   if (rc == SV_OK) rc = upload(b, host_states);
@@ -493,11 +533,15 @@ int sv_batch_read(sv_batch* b, int64_t run, double* host_soa, double* t, int64_t
     const size_t es = (size_t)b->esize;
     const size_t bytes = (size_t)(4 * st) * es;
     std::vector<unsigned char> pageable;
-    if (!b->staging) pageable.resize(bytes);
-    unsigned char* const tmp = b->staging ? b->staging : pageable.data();
-    const char* src = (const char*)b->buf[d.cur ? 1 : 0] + (size_t)d.off * es;
-    SVB_TRY(cudaMemcpyAsync(tmp, src, bytes, cudaMemcpyDeviceToHost, b->stream));
-    SVB_TRY(cudaStreamSynchronize(b->stream));
+    const unsigned char* tmp = b->staging + (b->whole ? (size_t)d.off * es : 0);
+    if (!b->whole) {
+      if (!b->staging) pageable.resize(bytes);
+      unsigned char* const to = b->staging ? b->staging : pageable.data();
+      const char* src = (const char*)b->buf[d.cur ? 1 : 0] + (size_t)d.off * es;
+      SVB_TRY(cudaMemcpyAsync(to, src, bytes, cudaMemcpyDeviceToHost, b->stream));
+      SVB_TRY(cudaStreamSynchronize(b->stream));
+      tmp = to;
+    }
     const double* ref = b->ps ? d.kp.ref : nullptr;
     if (es == 8) unpack_state((const double*)tmp, n, st, ref, host_soa);
     else unpack_state((const float*)tmp, n, st, ref, host_soa);
