@@ -80,7 +80,9 @@ def traffic_of(workload: str, ncell: int, precision: str, config: str):
 # of 8192^2; 3D 1575.8 counted with 60-plane segments, x (520/512) / (186/180) for the 128-plane
 # segments of 512^3).  With the paper's closure exponents (tau_rho = -1,
 # tau_T = -1.5: the power laws of eq. 6 as products).  These kernels are bound by GB300's FP64 pipe
-# (ncu: 86 % of its peak busy), so FP64 lines report an "alu" roofline.
+# (ncu: 86 % of its peak busy), so FP64 lines report an "alu" roofline.  The counts are those of the
+# step as first written, the work that an update stands for: the present kernels (sv_f64.cuh) do the
+# same update in fewer FP64 instructions, so "achieved" is the rate at which that work gets done.
 FP64_FLOPS_PER_CELL = {1: 422.9, 2: 775.5, 3: 1548.8}
 
 # --precision names -> sv_params.precision (SV_FP32, SV_FP64, SV_FP32_P64,
