@@ -359,9 +359,10 @@ int sv_batch_get_config(sv_batch* b, int* index, char* desc, size_t cap);
    field-major rho, rho v, E, E_nu; buffers sharing any byte return
    SV_EINVAL), with dt from eq. 16 (capped by c_tau * min tau) on U_in.  The
    same dt and, bit for bit, the same state as sv_step on a solver holding
-   U_in: it runs the sliding-warp kernel, whose per-cell arithmetic every 1D
-   kernel of the solver shares.  Allocates nothing and calls no allocating
-   routine.
+   U_in: every 1D kernel of the solver shares the per-cell arithmetic (grids of
+   up to 9600 float or 1792 double cells take one launch of one cluster, larger
+   ones a reset, a dt reduction and the sliding-warp step).  Allocates nothing
+   and calls no allocating routine.
    dt_used / flags (host pointers, each may be NULL) receive the dt taken and
    the SV_FLAG_* bits of the step; giving either makes the call wait for the
    stream, otherwise it is asynchronous on cuda_stream.
