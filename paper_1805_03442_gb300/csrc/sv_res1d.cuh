@@ -144,7 +144,9 @@ res1d_kernel(const KParams kp, R* bufA, R* bufB, Ctl* ctl, uint64_t* words, int 
 
   if (threadIdx.x == 0) {
     S.word[0] = S.word[1] = 0.0f;
-    S.stall = 0;
+    // read by one thread: a block that has started already may raise it meanwhile,
+    // and all threads of this one have to leave or stay together
+    S.stall = (vload(&ctl->flags) & FLAG_STALL) != 0;
   }
   // words by parity: block i's mailbox has NM bounds from each block (a private
   // one: polled by block i alone, so that no line is read by every SM), and
@@ -163,7 +165,7 @@ res1d_kernel(const KParams kp, R* bufA, R* bufB, Ctl* ctl, uint64_t* words, int 
     __threadfence();
   }
   const StepCtl sc = block_step_ctl(ctl);       // ends with a block barrier
-  if (!(sc.dt > 0.0) || (vload(&ctl->flags) & FLAG_STALL)) return;
+  if (!(sc.dt > 0.0) || S.stall) return;
   R* const U = sc.cur ? bufB : bufA;
   const P<R> k(kp);
   Clock<R> ck;
