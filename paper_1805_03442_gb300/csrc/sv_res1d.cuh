@@ -411,7 +411,9 @@ res1d_kernel(const KParams kp, R* bufA, R* bufB, Ctl* ctl, uint64_t* words, int 
     ctl->dt_cfl = (double)ck.dt_cfl;
     ctl->nsteps = nsteps0 + done;
     ctl->last = ck.last ? 1u : 0u;
-    ctl->flags = ck.flags;
+    // 0 when the launch began; a block that gave up in the last step has left its
+    // cells unwritten and may have raised its flag already
+    if (ck.flags) atomicOr(&ctl->flags, ck.flags);
     ctl->gen = sc.gen + 1u;         // every block has read it: each published a step
     set_step_dt<R>(ctl, ck.last ? ck.dt_last : (double)ck.dt, kp);
   }

@@ -45,3 +45,28 @@ def test_blocks_that_start_late(sv, prec, N):
         s.step(4)
         U, tu = s.read_state()
         assert s.status() == 0 and tu == t and np.array_equal(U, want)
+
+
+@pytest.mark.parametrize("prec, N, k", [("FP32", 4000, 2), ("FP32", 4000, 3), ("FP64", 1600, 1), ("FP64", 1600, 2)])
+def test_stall_of_the_last_step_is_kept(sv, prec, N, k):
+    """Runs of few steps with waits of few polls: a block that gives up in the last
+    step leaves its cells unwritten while the others finish.  The stall flag
+    stays, or the state, time and step count are those of per-step launches."""
+    P = sv.Params(precision=getattr(sv, prec), tau0=0.3)
+    U0 = inputs.random_states(1, N, seed=N, smooth=True)
+    want, t = per_step(sv, P, N, U0, k)
+    seen = set()
+    with sv.Solver(P, (N,), (1.0,)) as s:
+        s.set_launch(sv.LAUNCH_PERSISTENT)
+        for polls in (1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 64, 256, 4096):
+            s.set_wait_limit(polls)
+            for _ in range(30):
+                s.write_state(U0)
+                s.step(k)
+                U, tu = s.read_state()
+                bad = s.status()
+                seen.add(bad)
+                if not bad & sv.FLAG_STALL:
+                    assert bad == 0 and tu == t and s.time()[1] == k
+                    assert np.array_equal(U, want), (polls, int((U != want).any(axis=0).sum()))
+    assert sv.FLAG_STALL in seen and 0 in seen
