@@ -168,9 +168,12 @@ int sv_step(sv_solver* s, int64_t nsteps);
 /* How the steps of a solver are launched (sv_set_launch).
    SV_LAUNCH_PER_STEP: one kernel launch per step (two for SV_HEUN), replayed
      from a CUDA graph of 32 steps.
-   SV_LAUNCH_PERSISTENT: 1D MUSCL-Hancock only -- one launch runs up to 65536
-     steps, its blocks resident throughout, exchanging cells and dt bounds
-     after every step.  Bitwise the same results as per-step launches.
+   SV_LAUNCH_PERSISTENT: 1D MUSCL-Hancock only -- one launch runs up to 1024
+     steps (65536 on grids beyond the device's registers), its blocks resident
+     throughout, exchanging cells and dt bounds after every step.  Bitwise the
+     same results as per-step launches.  On a large grid the launch fills every
+     SM: kernels of other streams wait for its end (5 ms in float, 18 ms in double
+     at the most).
      Every wait gives up after about 2 s with SV_FLAG_STALL, which sv_run_to
      reports as SV_ESTALL.
    SV_LAUNCH_AUTO (default): persistent for 1D MUSCL-Hancock grids of at most

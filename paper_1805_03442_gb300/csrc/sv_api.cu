@@ -64,7 +64,14 @@ namespace {
 
 constexpr size_t kAlign = 256;
 constexpr int kGraphLen = 32;
-constexpr int64_t kLoopChunk = 1 << 16;   // steps per persistent launch at most
+constexpr int64_t kLoopChunk = 1 << 16;   // steps per sliding-loop launch, and per wait, at most
+// Steps per resident launch.  A launch on a large grid fills every SM's registers,
+// so kernels of other streams run between launches only: after at most 5 ms at 182000
+// float cells, 18 ms in double (65536 steps: 0.34 and 1.2 s).  Shorter launches cost a
+// launch and a read of the state each; us per step at 1024 / 65536 steps per launch:
+// 10^5 float cells 3.772 / 3.764, 1000 cells 2.606 / 2.603, 182000 in the
+// perturbation layout 5.208 / 5.194, 30000 double 17.92 / 17.92.
+constexpr int64_t kResChunk = 1 << 10;
 
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
@@ -264,7 +271,7 @@ int issue_steps(sv_solver* s, int64_t n) {
   if (n <= 0) return SV_OK;
   if (use_resident(s, n)) {
     while (n > 0) {
-      const int64_t m = n < kLoopChunk ? n : kLoopChunk;
+      const int64_t m = n < kResChunk ? n : kResChunk;
       SV_TRY(res1d_launch(s->p.precision, s->kp, s->buf[0], s->buf[1], s->ctl, s->res_words,
                           s->ncell, s->res, (int)m, s->stream));
       n -= m;
@@ -531,9 +538,15 @@ int sv_run_to(sv_solver* s, double t_end, int64_t max_steps, int64_t* steps_take
     double est = ceil((t_end - c.t) / (c.dt_cfl > 0.0 ? c.dt_cfl : c.dt));
     if (!(est >= 1.0)) est = 1.0;
     int64_t n = est > 1e15 ? (int64_t)1e15 : (int64_t)est;
-    n = n > 4096 ? 4096 : n;
-    // the persistent loops stop by themselves at t_end: no estimate needed
-    if (use_loop(s) || use_resident(s, n)) n = kLoopChunk;
+    if (use_resident(s, n)) {
+      // a launch stops by itself at t_end: one needs no estimate, and of several
+      // those behind the end return at once
+      n = n < kResChunk ? kResChunk : (n < kLoopChunk ? n : kLoopChunk);
+    } else if (use_loop(s)) {
+      n = kLoopChunk;
+    } else if (n > 4096) {
+      n = 4096;
+    }
     if (n > max_steps - done) n = max_steps - done;
     if (n < 1) n = 1;
     rc = issue_steps(s, n);
