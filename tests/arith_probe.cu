@@ -9,7 +9,10 @@ namespace {
 
 __global__ void f64_kernel(int op, const double* x, double* y, int n) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) y[i] = op == 0 ? d64::rcp(x[i]) : d64::sqrt_pos(x[i]);
+  if (i >= n) return;
+  if (op == 0) y[i] = d64::rcp(x[i]);
+  else if (op == 1) y[i] = d64::sqrt_pos(x[i]);
+  else y[i] = op == 2 ? d64::rcp_estimate(x[i]) : d64::rsqrt_estimate(x[i]);
 }
 
 // p of (kin2, E, E_nu) by the scalar and by the packed recovery, two states a thread
@@ -43,7 +46,7 @@ int with_buffers(const void* in, size_t nin, void* out, size_t nout, F&& go) {
 
 }  // namespace
 
-// op 0: d64::rcp, 1: d64::sqrt_pos of n doubles.
+// op 0: d64::rcp, 1: d64::sqrt_pos, 2 and 3: the estimates they begin with, of n doubles.
 extern "C" int probe_f64(int op, const double* x, double* y, int n) {
   return with_buffers(x, sizeof(double) * n, y, sizeof(double) * n, [&](void* a, void* b) {
     f64_kernel<<<(n + 255) / 256, 256>>>(op, (const double*)a, (double*)b, n);
