@@ -70,9 +70,10 @@ extern "C" {
 #define SV_FP32     0   /* float state and arithmetic */
 #define SV_FP64     1   /* double state and arithmetic */
 #define SV_FP32_P64 2   /* float state, pressure recovery of eq. 5 to double accuracy: the
-                           exact E - rho v^2/2 - E_nu of the float operands, times
-                           gamma - 1 held to ~2^-48, rounded once (within the last bit of
-                           the subtraction carried out in double) */
+                           exact E - rho v^2/2 - E_nu of the float operands (E_nu >= -E),
+                           times gamma - 1 held to ~2^-48, rounded once (within the last
+                           bit of the subtraction carried out in double).  No double
+                           instruction is spent on it: a pair of floats holds the sum */
 #define SV_FP32_PC  3   /* the same arithmetic (two error-free float sums) under the name of
                            the compensated-float policy, with that policy's choice of
                            launch configurations */

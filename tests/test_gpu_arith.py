@@ -1,6 +1,8 @@
 """The step kernels' own arithmetic, function by function on the device
 (tests/arith_probe.cu): the reciprocal and square root of the double kernels
-(csrc/sv_f64.cuh) against the exact results, with the bound that the series gives."""
+(csrc/sv_f64.cuh) and the pressure recovery of SV_FP32_P64 / SV_FP32_PC
+(pressure<2> of csrc/sv_model.cuh, packed in csrc/sv_pair1d.cuh), each against
+64 bits with the bound that its series or its sums give."""
 import ctypes
 import os
 import subprocess
@@ -13,6 +15,7 @@ from gpu_util import need_gpu
 pytestmark = pytest.mark.gpu
 
 HERE = os.path.dirname(os.path.abspath(__file__))
+f32, f64 = np.float32, np.float64
 
 
 @pytest.fixture(scope="module")
@@ -90,3 +93,57 @@ def test_square_root(probe):
     err = np.abs((x - p) - q) / (2.0 * y) / np.spacing(y)
     print(f"estimate 2^{np.log2(e):.2f}, square root {err.max():.4f} ulp")
     assert err.max() <= 0.5 + 11 / 16 * 2.0 ** 53 * e ** 3 + 2.0 ** -16
+
+
+def pressures(probe, gamma, kin2, E, Ev):
+    s = np.ascontiguousarray(np.stack([kin2, E, Ev]))
+    p = np.empty((2, len(E)), f32)
+    probe.probe_pressure.argtypes = [ctypes.c_double, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int]
+    assert probe.probe_pressure(gamma, ptr(s), ptr(p), len(E)) == 0
+    return p
+
+
+def states(seed, ev, n=400_000):
+    rng = np.random.default_rng(seed)
+    kin2 = (10.0 ** rng.uniform(-12, 2, n) * rng.integers(0, 2, n)).astype(f32)
+    p = rng.uniform(1e-3, 4.0, n)
+    Ev = ev * rng.uniform(0.5, 2.0, n)
+    E = (p / 0.4 + 0.5 * kin2 + np.maximum(Ev, 0.0)).astype(f32)
+    if ev < 0:                            # E_nu between -E and 0
+        Ev = -E * rng.uniform(0.0, 1.0, n)
+    return kin2, E, Ev.astype(f32)
+
+
+@pytest.mark.parametrize("gamma", [1.4, 5 / 3, 1.05])
+@pytest.mark.parametrize("ev", [-1.0, 0.0, 0.1, 1.0, 30.0, 1000.0])
+def test_pressure_without_a_rounding_before_the_last(probe, gamma, ev):
+    """gamma - 1 times the difference that double carries out, rounded once: what
+    is rounded before is 2^-24 of e1 + e2 (themselves 2^-24 of the sums s and t)
+    and of the small part of gamma - 1.  The packed recovery gives the same bits."""
+    kin2, E, Ev = states(int(10 * ev) + 20, ev)
+    q = E.astype(f64) - 0.5 * kin2.astype(f64) - Ev.astype(f64)
+    ok = q > 0
+    assert ok.mean() > 0.9
+    one, two = pressures(probe, gamma, kin2, E, Ev)
+    assert np.array_equal(one, two)
+    want = (gamma - 1.0) * q[ok]
+    ulp = np.spacing(want.astype(f32)).astype(f64)
+    s = np.abs(E.astype(f64) - Ev)[ok]
+    err = np.abs(one[ok].astype(f64) - want) / ulp
+    assert np.all(err <= 0.5 + 2.0 ** -22 * (1.0 + s / q[ok]))
+    # the double policy's own rounding of the same number: its last bit at most
+    assert np.all(np.abs(one[ok].astype(f64) - want.astype(f32)) <= ulp)
+
+
+def test_sign_of_p_is_exact(probe):
+    """States around and below p = 0, where the guard decides on the sign."""
+    rng = np.random.default_rng(9)
+    n = 400_000
+    Ev = (10.0 ** rng.uniform(-3, 3, n)).astype(f32)
+    h = 10.0 ** rng.uniform(-6, 3, n)
+    E = (Ev + h * rng.choice([0.0, 0.5, 1.0, 1.0 + 1e-7, 1.0 - 1e-7, 2.0], n)).astype(f32)
+    E = np.where(rng.random(n) < 0.1, (0.9 * Ev).astype(f32), E)
+    kin2 = (2.0 * h).astype(f32)
+    q = E.astype(f64) - 0.5 * kin2.astype(f64) - Ev.astype(f64)
+    for p in pressures(probe, 1.4, kin2, E, Ev):
+        assert np.array_equal(np.sign(p), np.sign(q))
