@@ -464,8 +464,8 @@ int sv_init(const sv_params* p, const sv_grid* g, void* cuda_stream, void* devic
   }
   if (rc == SV_OK && s->dim == 1 && p->method == SV_HANCOCK) {
     // 0 where the device has no cooperative launch: the per-step path remains
-    int dev = 0, sms = 0, cap = 0;
-    s->loop_grid = loop1d_grid(s->kp, p->precision, s->ncell, &cap);
+    int dev = 0, sms = 0;
+    s->loop_grid = loop1d_grid(s->kp, p->precision, s->ncell);
     if (cudaGetDevice(&dev) == cudaSuccess)
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     s->res = res1d_shape(s->kp, p->precision, s->ncell);
@@ -688,7 +688,9 @@ int sv_set_launch(sv_solver* s, int mode) {
 
 int sv_set_wait_limit(sv_solver* s, int polls) {
   if (!s || polls < 0) return SV_EINVAL;
-  s->kp.stall_polls = polls;   // read by the persistent loop only, which is never captured
+  // read by the persistent loops only, as a launch argument: a launch captured
+  // before keeps the limit it was captured with
+  s->kp.stall_polls = polls;
   return SV_OK;
 }
 

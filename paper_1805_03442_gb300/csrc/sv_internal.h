@@ -47,7 +47,7 @@ cudaError_t tile1d_launch(const KParams& kp, int precision, int var, void* a, vo
                           int64_t N, int grid, cudaStream_t st, bool pdl = false);
 
 // 1D persistent loop of up to nmax steps (sv_loop1d.cu); grid 0 = unavailable
-int loop1d_grid(const KParams& kp, int precision, int64_t N, int* cap);
+int loop1d_grid(const KParams& kp, int precision, int64_t N);
 cudaError_t loop1d_launch(int precision, const KParams& kp, void* a, void* b, Ctl* ctl, int64_t N,
                           int grid, int64_t nmax, cudaStream_t st);
 

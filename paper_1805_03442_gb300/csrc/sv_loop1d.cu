@@ -1,11 +1,10 @@
 // sv_loop1d.cu -- many 1D MUSCL-Hancock steps (Sec. 2.3: eqs. 13-15 with
 // xi = 0, source Y, eq. 16 reduction) in one persistent launch.
 //
-// On the grids of the paper's own experiments (a few hundred to 10^5 cells)
-// one step is a chain of latencies -- loading a chunk, three sliding
-// iterations of one warp, the block fold and the serial dt finalize -- rather
-// than a throughput problem, and a kernel boundary per step adds to it.  This
-// kernel keeps its blocks resident for a whole run of steps instead:
+// The persistent mode of the grids that the resident loop (sv_res1d.cuh) does not
+// hold: above 182400 cells in float and 34048 in double on 152 SMs, and the grid of
+// one cell.  A step's fixed part (the launch, the block fold and the serial dt
+// finalize) is paid by a grid-wide barrier here in place of a kernel boundary:
 //   - every block computes its chunks of the step with the same per-warp body
 //     as the one-step kernel (sv_step1d.cuh), so each cell gets the same
 //     operations in the same order and the results are bitwise equal;
@@ -147,18 +146,14 @@ size_t smem_bytes(int precision) {
 
 }  // namespace
 
-// Grid of the persistent loop for N cells: one block per 64-cell chunk while
-// the device holds that many, so that the few busy warps of a small grid sit
-// on different SMs (each warp's critical path is its own chunk; in double the
-// SM's FP64 pipe, not latency, bounds it); beyond that as many blocks as fit
-// at once, every warp sliding over several chunks.  Sets the kernel's
+// Grid of the persistent loop for N cells: as many blocks as fit at once, every
+// warp sliding over several chunks; never more than chunks.  Sets the kernel's
 // shared-memory limit (host side, outside any capture).  Returns 0 if the
-// device cannot launch it cooperatively; *cap receives the co-resident limit.
-int loop1d_grid(const KParams& kp, int precision, int64_t N, int* cap) {
+// device cannot launch it cooperatively.
+int loop1d_grid(const KParams& kp, int precision, int64_t N) {
   int dev = 0, sms = 0, per = 0, coop = 0;
   const void* fn = pick(kp, precision);
   const size_t smem = smem_bytes(precision);
-  if (cap) *cap = 0;
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
@@ -168,7 +163,6 @@ int loop1d_grid(const KParams& kp, int precision, int64_t N, int* cap) {
   if (!coop || per < 1 || sms < 1) return 0;
   const int64_t want = (N + 63) / 64;
   const int64_t limit = (int64_t)sms * per;
-  if (cap) *cap = (int)limit;
   return (int)(want < limit ? (want < 1 ? 1 : want) : limit);
 }
 
