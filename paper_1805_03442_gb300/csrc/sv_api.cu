@@ -696,7 +696,7 @@ int sv_set_wait_limit(sv_solver* s, int polls) {
 
 int sv_get_launch(sv_solver* s, int* mode) {
   if (!s || !mode) return SV_EINVAL;
-  *mode = use_loop(s) ? SV_LAUNCH_PERSISTENT : SV_LAUNCH_PER_STEP;
+  *mode = use_loop(s) || use_resident(s, 1) ? SV_LAUNCH_PERSISTENT : SV_LAUNCH_PER_STEP;
   return SV_OK;
 }
 
