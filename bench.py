@@ -81,9 +81,15 @@ def traffic_of(workload: str, ncell: int, precision: str, config: str):
 # segments of 512^3).  With the paper's closure exponents (tau_rho = -1,
 # tau_T = -1.5: the power laws of eq. 6 as products).  These kernels are bound by GB300's FP64 pipe
 # (ncu: 86 % of its peak busy), so FP64 lines report an "alu" roofline.  The counts are those of the
-# step as first written, the work that an update stands for: the present kernels (sv_f64.cuh) do the
-# same update in fewer FP64 instructions, so "achieved" is the rate at which that work gets done.
+# step as first written, the work that an update stands for: "achieved" and "frac" are the rate at
+# which that work gets done, not the use of the pipe.  The present kernels (sv_f64.cuh) do the same
+# update in the operations of FP64_EXECUTED_PER_CELL, counted the same way on the same grids (2D
+# 582.6 with 96-row segments, x (1 + 1.2/256) / (1 + 1.2/96); 3D 1250.1 with 26-plane segments,
+# x (1 + 1.2/64) / (1 + 1.2/25.7): a segment's two extra planes cost 1.2); "executed" reports
+# those.  A DMUL or DADD slot carries one of them, a DFMA two, so that a pipe busy 86 % of the time
+# reads 0.6 there.
 FP64_FLOPS_PER_CELL = {1: 422.9, 2: 775.5, 3: 1548.8}
+FP64_EXECUTED_PER_CELL = {1: 284.8, 2: 578.1, 3: 1216.7}
 
 # --precision names -> sv_params.precision (SV_FP32, SV_FP64, SV_FP32_P64,
 # SV_FP32_PC, SV_FP32_PS of include/sv.h) and the arithmetic type reported as "dtype"
@@ -92,14 +98,19 @@ DTYPES = {"fp32": "f32", "fp64": "f64", "fp32_p64": "f32", "fp32_pc": "f32", "fp
 
 
 def fp64_roofline(dim: int, ncell: int, step_s: float, hbm_frac: float, peak: float) -> dict:
-    """The FP64 step as an ALU-bound kernel: FP64 flops per launch
+    """The FP64 step as an ALU-bound kernel: the update's FP64 work per launch
     (FP64_FLOPS_PER_CELL) over the FP64 FMA rate the library's probe measured
-    in this run (`peak`, TFLOP/s)."""
+    in this run (`peak`, TFLOP/s); `executed`: the same of the operations that
+    the kernel executes for it (FP64_EXECUTED_PER_CELL)."""
     flops = FP64_FLOPS_PER_CELL[dim] * ncell
     achieved = flops / step_s / 1e12
+    executed = FP64_EXECUTED_PER_CELL[dim] * ncell / step_s / 1e12
     return {"bound": "alu", "achieved": achieved, "peak": peak,
             "peak_src": "measured: DFMA-chain probe of the library (sv_measure_fp64_peak), this run",
             "unit": "TFLOP/s", "frac": achieved / peak, "traffic": None,
+            "counts": "achieved, frac: work of the update as first written; executed: operations of the kernel",
+            "executed": {"flops_per_cell": FP64_EXECUTED_PER_CELL[dim], "achieved": executed,
+                         "frac": executed / peak},
             "flops_per_launch": flops, "hbm_frac": hbm_frac}
 
 
