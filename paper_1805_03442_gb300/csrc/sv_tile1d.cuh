@@ -80,6 +80,17 @@ __device__ __forceinline__ void copy_interior(float (*dst)[SPAN], const float* U
   if (q == 0) cp16(d + 4 * (C4 - 1), src + 4 * (C4 - 1));
 }
 
+// The ghost cell's state out of line, for the float policy: two cells of one tile
+// need it, and its exp and sincos inside the tile loop displace the registers and
+// the schedule of everything else.  us per step inlined / called: 2^22 cells 42.71 /
+// 41.97, 2^24 154.7 / 151.3; driven at 2^20 cells 13.76 / 13.57, at 65536 (single
+// steps; longer runs are resident) 6.68 / 7.05.  The other policies keep it inline
+// (compensated 48.7 either way, perturbations 52.7 and driven 7.32 / 7.63).
+static __device__ __noinline__ void drive_state_call(const KParams& kp, double x, double t,
+                                                     double (&u)[4]) {
+  drive_state(kp, x, t, u);
+}
+
 template <int SPAN, int PP, int NT>
 __device__ __forceinline__ void load_tile(float (*dst)[SPAN], const float* Uin, int N, int b,
                                           const P<float>& k, const KParams& kp, double t) {
@@ -91,7 +102,8 @@ __device__ __forceinline__ void load_tile(float (*dst)[SPAN], const float* Uin, 
       const int j = lo + e;
       if (j < 0 && k.bc_lo == BC_DRIVEN) {
         double u[4];
-        drive_state(kp, ((double)j + 0.5) * kp.h, t, u);
+        if constexpr (PP == 0) drive_state_call(kp, ((double)j + 0.5) * kp.h, t, u);
+        else drive_state(kp, ((double)j + 0.5) * kp.h, t, u);
 #pragma unroll
         for (int f = 0; f < 4; ++f) dst[f][e] = (float)(PP == 3 ? u[f] - kp.ref[f] : u[f]);
       } else {
