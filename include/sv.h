@@ -196,13 +196,12 @@ int sv_set_launch(sv_solver* s, int mode);
    SV_LAUNCH_PERSISTENT; AUTO resolved). */
 int sv_get_launch(sv_solver* s, int* mode);
 
-/* Bound of the persistent loop's grid-barrier waits, for exercising its
-   failure path: every wait gives up after `polls` polls of the barrier
-   generation (or the ~2 s time limit, whichever comes first); 0 (the default)
-   restores the limit of 2^24 polls.  A wait that gives up raises
-   SV_FLAG_STALL and leaves the launch, so sv_step / sv_run_to end with
-   SV_ESTALL and the state is undefined until the next sv_write_state (which
-   also clears the flag).  Per-step launches do not wait and ignore it.
+/* Bound of the persistent loops' waits, for exercising their failure path: every
+   wait for another block gives up after `polls` polls (or the ~2 s time limit,
+   whichever comes first); 0 (the default) restores the limit of 2^24 polls.  A
+   wait that gives up raises SV_FLAG_STALL and leaves the launch, so sv_run_to
+   ends with SV_ESTALL and the state is undefined until the next sv_write_state
+   (which also clears the flag).  Per-step launches do not wait and ignore it.
    Errors: SV_EINVAL (null solver, polls < 0). */
 int sv_set_wait_limit(sv_solver* s, int polls);
 
@@ -218,13 +217,17 @@ int sv_set_wait_limit(sv_solver* s, int polls);
  *     axis (fewer where a small grid would otherwise not fill the device).
  * sv_autotune times each configuration on the solver's current state and
  * keeps the fastest; the state, time and status are restored afterwards.
+ * Runs that the resident launches take do not use the per-step kernel: on a 1D
+ * grid that fits in the device's registers (182400 float cells on a GB300) in
+ * mode SV_LAUNCH_AUTO, the choice concerns single float steps only, and in
+ * SV_LAUNCH_PER_STEP all steps (sv_set_launch).
  * ------------------------------------------------------------------------ */
 
 /* Number of launch configurations of this solver (>= 1). */
 int sv_num_configs(sv_solver* s, int* count);
 
-/* Current configuration index and its description (desc may be NULL;
-   truncated to cap bytes including the terminating zero). */
+/* Current configuration index of the per-step kernel and its description (desc
+   may be NULL; truncated to cap bytes including the terminating zero). */
 int sv_get_config(sv_solver* s, int* index, char* desc, size_t cap);
 
 /* Description of configuration `index`. */

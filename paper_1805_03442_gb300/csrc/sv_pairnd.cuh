@@ -69,8 +69,8 @@ __device__ __forceinline__ void add_dflux(const f2 (&d)[DIM + 3], const f2 (&a)[
 // (27 packed operations in 2D instead of 30).  The mass flux keeps the momenta
 // themselves, the normal momentum its whole flux (the pressures gathered first
 // would round the sum at the size of p twice more: 1000 x 700 cells, 16 steps, error
-// against 64 bits 1.01e-7 with the flux, 1.20e-7 so; the same operation count and
-// time), and the difference its own weight: folding wd into the weights of L and R
+// against 64 bits 9.35e-8 with the flux, 1.106e-7 so; the same operation count, and
+// 8192^2 at 1186 and 1185 us), and the difference its own weight: folding wd into the weights of L and R
 // would cancel terms of the size of c u.
 template <int DIM, int A>
 __device__ __forceinline__ void hll_sum(const f2 (&L)[DIM + 3], const f2 (&R)[DIM + 3], f2 wl, f2 wr,

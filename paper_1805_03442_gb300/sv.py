@@ -388,7 +388,7 @@ class Solver:
 
     @property
     def launch(self) -> int:
-        """The launch mode the next steps use (LAUNCH_PER_STEP or LAUNCH_PERSISTENT)."""
+        """The launch mode a single next step uses (LAUNCH_PER_STEP or LAUNCH_PERSISTENT)."""
         m = ctypes.c_int()
         _check(lib().sv_get_launch(self._h, ctypes.byref(m)), "sv_get_launch")
         return m.value
@@ -416,9 +416,10 @@ class Solver:
         _check(lib().sv_set_config(self._h, int(index)), "sv_set_config")
 
     def autotune(self, steps: int = 10, cold: bool = False) -> tuple[int, list[float]]:
-        """Time every configuration on the current state (restored after each
-        trial) and keep the fastest; cold: each timed step after an L2-evicting
-        write.  Returns (index, microseconds per step of each configuration)."""
+        """Time every configuration of the per-step kernel on the current state
+        (restored after each trial) and keep the fastest; cold: each timed step after
+        an L2-evicting write.  Runs in resident launches (sv_set_launch) do not use
+        it.  Returns (index, microseconds per step of each configuration)."""
         n = len(self.configs())
         us = (ctypes.c_double * n)()
         best = ctypes.c_int()

@@ -12,6 +12,10 @@ Cache layout::
 
     {"<device>": {"<key>": {"config": "<description>", "us": [..], "when": <unix time>}}}
 
+What is tuned is the per-step kernel: 1D runs of several steps on grids that fit
+in the device's registers take the resident launches in the default launch mode,
+whatever is chosen here.
+
 The description, not the index, is stored: if the library's list of
 configurations changes, a stale entry no longer matches and is tuned again.
 """
