@@ -533,13 +533,8 @@ def precision_leg(sv, args, prec_name: str, U0, dims, L, stream, flush, pk: dict
            "status_flags": status}
     if prec == sv.FP64:
         peak = sv.measure_fp64_peak(stream)
-        flops = FP64_FLOPS_PER_CELL[len(dims)] * ncell
-        out["roofline"] = {"bound": "alu", "achieved": flops / step_s / 1e12, "peak": peak,
-                           "peak_src": "measured: DFMA-chain probe of the library "
-                                       "(sv_measure_fp64_peak), this run",
-                           "unit": "TFLOP/s", "frac": flops / step_s / 1e12 / peak,
-                           "traffic": None, "flops_per_launch": flops,
-                           "hbm_frac": alg / step_s / 1e9 / pk["hbm_gbs"]}
+        out["roofline"] = fp64_roofline(len(dims), ncell, step_s, alg / step_s / 1e9 / pk["hbm_gbs"],
+                                        peak)
         out["error_vs_oracle"] = fp64_sampled_parity(sv, P, dims, L, U0)
     else:
         out["roofline"] = {"bound": "hbm", "achieved": alg / step_s / 1e9, "peak": pk["hbm_gbs"],

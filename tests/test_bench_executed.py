@@ -1,5 +1,6 @@
 """The FP64 roofline's executed operations (no GPU): the kernels' own rate next to
 that of the work an update stands for."""
+import inspect
 import os
 import sys
 
@@ -19,3 +20,8 @@ def test_executed_is_what_the_pipe_can_do(dim, ncell, step_s):
     assert e["frac"] == pytest.approx(e["achieved"] / r["peak"])
     assert e["flops_per_cell"] < bench.FP64_FLOPS_PER_CELL[dim]
     assert 0.5 < e["frac"] < 0.86
+
+
+def test_every_fp64_line_reports_it():
+    """The lines of the benchmark that have an ALU roofline all take it from there."""
+    assert inspect.getsource(bench).count('"bound": "alu"') == 1
