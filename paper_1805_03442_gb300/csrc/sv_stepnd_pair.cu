@@ -422,9 +422,10 @@ stepnd_pair_kernel(const KParams kp, float* __restrict__ bufA, float* __restrict
 }
 
 // Tiles of the pair kernel: 128 threads along x (126 interior cells), 162-168
-// registers, 3 blocks per SM (a budget of 4 spills).  It is bound by the issue
-// slots and the FMA pipe its packed operations hold for two cycles each
-// (profiles/stepnd2d_fp32_4096x4096.md): folding the fluxes into the sums that use
+// registers, 3 blocks per SM (a budget of 4 spills).  No unit is full
+// (issue slots 57 % of the cycles, the FMA pipe, which a packed operation holds for
+// two, 51 %; profiles/stepnd2d_fp32_4096x4096.md): three warps per scheduler wait on
+// fixed latencies, shared memory and three barriers per row pair.  Folding the fluxes into the sums that use
 // them and the 32-bit offsets took 8192^2 from 1227 to 1185 us per step (FP32;
 // 2000 x 1500 in compensated float 80.6 -> 77.0).  192 threads x 2 blocks 1259 us,
 // 96 x 4 1224 (1000 x 1000 with walls 45.9 -> 63.8); the transverse fluxes left in
