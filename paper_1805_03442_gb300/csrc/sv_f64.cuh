@@ -301,7 +301,8 @@ __device__ __forceinline__ void bound(const P<double>& k, const double (&u)[DIM 
   const float sf = fmaxf(2.0f * vf, vf + cf) * (1.0f + 0x1p-18f);
   if (!(ok && sf < s)) {
     const double vm = DIM == 1 ? v2 : (v2 > 0x1p-1000 ? sqrt_pos(v2) : 0.0);
-    const double c = sqrt_pos(c2);
+    // where it overflows the speed is infinite (dt is then flagged), not inf * 0
+    const double c = __double2hiint(c2) < 0x7ff00000 ? sqrt_pos(c2) : c2;
     const double sx = fmax(add(vm, vm), add(vm, c));
     m.smax = fmax(m.smax, sx);
     bool fits = true;

@@ -353,8 +353,11 @@ __device__ __forceinline__ bool all_positive(double a, double b, double c, doubl
   return min(min(ha, hb), min(hc, hd)) > 0;
 }
 __device__ __forceinline__ bool both_positive(float a, float b) { return (a > 0.0f) && (b > 0.0f); }
+// Double: positive and no NaN, whatever the NaN's sign (that of the SFU's estimates
+// is positive, CUDA's own negative): high words 1 .. 0x7ff00000 (infinity).
 __device__ __forceinline__ bool both_positive(double a, double b) {
-  return min(__double2hiint(a), __double2hiint(b)) > 0;
+  const unsigned x = (unsigned)__double2hiint(a) - 1u, y = (unsigned)__double2hiint(b) - 1u;
+  return (x > y ? x : y) < 0x7ff00000u;
 }
 
 // TVD slope limiters on the two one-sided differences a, b (eq. 14 asks for
